@@ -10,9 +10,10 @@
 //               when the tile lies in one active frame, else gathered by frame index in
 //               8-row boxes) and streams K/V tiles of 128 tokens through a ring of
 //               shared-memory slots.
-//   warp 1      owns TMEM (512 columns) and one lane issues every tcgen05.mma:
+//   warps 1, 2  issue the tcgen05.mma of query tile A and of query tile B:
 //               S = Q K^T (both operands in shared memory) and O += P V (P in TMEM).
-//   warp 2      (block-masked launches) builds each work item's list of KV tiles.
+//               Warp 1 owns TMEM (512 columns).
+//   warp 3      (block-masked launches) builds each work item's list of KV tiles.
 //   warps 4-7   softmax for query tile A, warps 8-11 for query tile B: thread = query row;
 //               online softmax in fp32 with base-2 exponentials, lazy rescaling of the O
 //               accumulator (only when the running max grows by more than 2^8), P rounded
@@ -20,12 +21,23 @@
 // TMEM columns: S_A [0,128), S_B [128,256), O_A [256,256+d), O_B [384,384+d); P_X aliases
 // the first 64 columns of S_X.
 //
-// MMA issue order per KV tile j (after the prologue S_A(0), S_B(0), PV_A(0)):
-//   S_A(j+1), PV_B(j), S_B(j+1), PV_A(j+1)
-// so each softmax group has one QK^T and one PV of the other group to hide behind.  Each
-// S_X(j+1) is committed after PV_X(j) was issued, so the softmax warps that wait for S_X(j+1)
-// also know that O_X is no longer being written and may rescale it in place.  Reuse of the
-// S/P columns by the next QK^T relies on tcgen05.mma operations issued by one thread
+// One KV step of a tile pair is the chain P_X(j) -> PV_X(j), S_X(j+1) -> softmax -> P_X(j+1) of
+// each tile, with the two GEMMs of one tile run by the tensor core while the other tile is in its
+// softmax.  At head dim 128 the four GEMMs take 2,100 cycles (measured alone: 560 for Q K^T, 512
+// for PV, 512 each when they alternate) and a tile's softmax about 1,100, so the step is bound by
+// the tensor core only if the hand-offs between the warps stay short.  What that took (cycles per
+// KV step, 13 x 1560 tokens x 12 heads, measured by the issuing warps without other probes):
+//   2767  one thread issuing for both tiles under a branch on the lane number
+//   2594  waits by the whole warp, MMAs by the thread that elect.sync picks, P handed over through
+//         named barriers and in two halves (head dim 64: 2606 -> 1956)
+//   2368  one issuing warp per tile, taking turns: a warp waits for its own P, K and V while the
+//         other warp's MMAs run, instead of behind them in one instruction stream
+//   2290  the turn taken before the wait for P, not after it
+// At 2290 the sustained rate of long launches is set by the power cap (1.67 GHz against 1.80 before).
+// Without the turns the two chains fall into step: both softmaxes at once, then both GEMM pairs
+// (4,300 cycles).  Each S_X(j+1) is committed after PV_X(j) was issued, so the softmax warps that
+// wait for S_X(j+1) also know that O_X is no longer being written and may rescale it in place.
+// Reuse of the S/P columns by the next QK^T relies on tcgen05.mma operations issued by one thread
 // executing in issue order.
 //
 // Work item = (head, pair of 128-row query tiles) over the flattened list of active rows
@@ -62,7 +74,25 @@ constexpr int kThreads = 384;  // three warpgroups
 constexpr int kRegsLaunch = 168, kRegsControl = 104, kRegsSoftmax = 200;
 static_assert(128 * kRegsControl + 256 * kRegsSoftmax <= kThreads * kRegsLaunch, "register split");
 constexpr uint32_t kTmemCols = 512;
-constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s: no legitimate wait comes close
+// P is handed to the tile's MMA warp in two parts, the first kPSplit keys and the rest: PV starts
+// on the first part while the softmax warps still compute the second.  These hand-offs, and the
+// turns of the two MMA warps, are hardware named barriers (an mbarrier takes 170-235 cycles longer
+// per hand-off between busy warps).  A named barrier has no time limit of its own, so who waits
+// on one is always released by others: only the MMA warps wait on them, every other wait of the
+// kernel is bounded and raises the abort flag on expiry, and a warp that gives up keeps arriving
+// on the barriers it owes (release_mma) until the waiting MMA warp, which reads the abort flag
+// in every round of its loop, has left.  All counts are multiples of a warp, so surplus arrivals
+// complete a barrier exactly.
+constexpr int kPSplit = 64;  // 32, 64, 96, 128: 2338, 2368, 2510, 2757 cycles per step
+constexpr int kPThreads = 128 + 32;
+__device__ __forceinline__ int p_barrier(int X, int part) { return 1 + 2 * X + part; }
+// The two MMA warps take turns; a turn is passed on before the last kTurnAhead MMAs of a group, so
+// that the other warp's MMAs follow without a gap (head dim 128: 0, 1, 2, 3, 4 measured within 1%;
+// head dim 64: 2051, 2081, 2130, 2212, 2230 cycles per step).
+template <int D>
+constexpr int kTurnAhead = D == 128 ? 2 : 0;
+__device__ __forceinline__ int turn_barrier(int X) { return 5 + X; }
+constexpr uint32_t kWaitLimitNs = 2000000000u;  // 2 s: no legitimate wait comes close
 constexpr uint64_t kDrainLimitNs = 200000000ull;  // 0.2 s for in-flight copies at teardown
 constexpr float kRescaleLog2 = 8.0f;
 constexpr int kMaxSplit = 16;          // KV ranges per split item
@@ -83,13 +113,13 @@ struct Cfg {
   static constexpr int kSlots = (D == 128) ? 4 : 8;
   static constexpr int kOffKV = 2 * kTileBytes;
   static constexpr int kOffBar = kOffKV + kSlots * kTileBytes;
-  // barriers: q_full[2] q_empty[2] kv_full[S] kv_empty[S] s_full[2] p_full[2] o_done[2]
+  // barriers: q_full[2] q_empty[2] kv_full[S] kv_empty[S] s_full[2] o_done[2]
   // group[2] (the 128 threads of one softmax warpgroup) drain
   static constexpr int kBarQFull = 0, kBarQEmpty = 2, kBarKVFull = 4, kBarKVEmpty = 4 + kSlots,
-                       kBarSFull = 4 + 2 * kSlots, kBarPFull = kBarSFull + 2,
-                       kBarODone = kBarPFull + 2, kBarGroup = kBarODone + 2,
-                       kBarDrain = kBarGroup + 2, kNumBars = kBarDrain + 1;
-  // misc: tmem address, abort flag, merge flags [2 groups][2 alternating slots]
+                       kBarSFull = 4 + 2 * kSlots, kBarODone = kBarSFull + 2, kBarGroup = kBarODone + 2,
+                       kBarDrain = kBarGroup + 2, kNumBars = kBarDrain + 2;
+  // misc: tmem address, abort flag, merge flags [2 groups][2 alternating slots],
+  // MMA warps done [2]
   static constexpr int kOffMisc = kOffBar + kNumBars * 8;
   static constexpr int kSmemBytes = kOffMisc + 32 + 1024;  // + slack to align the base
   // (MASKED) tile-list ring: barriers tl_full[kTLSlots] tl_empty[kTLSlots] tl_claim (+ 8 bytes
@@ -269,6 +299,12 @@ __device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity) {
     if (globaltimer_ns() - t0 > kDrainLimitNs) return;
 }
 
+// One arrival for the whole warp, after everything its lanes did before.
+__device__ __forceinline__ void warp_arrive(uint32_t bar) {
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+}
+
 // All 128 threads of one softmax warpgroup meet on an mbarrier (count 128); the wait is
 // bounded like every other wait and its result is warp-uniform.
 __device__ __forceinline__ bool group_sync(uint32_t bar, int& cnt, volatile int* abort) {
@@ -299,8 +335,8 @@ struct TLRing {
     return static_cast<int>(words(k)[kTLWords + 1]);
   }
 };
-// Arrivals that release a slot: the producer, the MMA issuer and the 256 softmax threads.
-constexpr int kTLConsumers = 2 + 256;
+// Arrivals that release a slot: the producer, the two MMA warps and the 256 softmax threads.
+constexpr int kTLConsumers = 3 + 256;
 // (work queue, at most kJitUnitsPerCta units per CTA) KV tiles of the current unit still to load
 // when the next unit is claimed.  A unit is then taken from the queue only when its CTA is about
 // to need it, so the queue's longest-first order decides which CTA gets which item as CTAs
@@ -321,7 +357,7 @@ __device__ __forceinline__ bool claim_jit(const AttnParams& p, const Sched& sc) 
 constexpr int kQueueNext = 0, kQueueDone = 1;
 
 // ---------------------------------------------------------------------------------------
-// Tile-list builder (MASKED only; warp 2, all 32 lanes).
+// Tile-list builder (MASKED only; warp 3, all 32 lanes).
 // ---------------------------------------------------------------------------------------
 // For every unit of this CTA, in order, one ring slot receives the bitmap of the KV tiles the
 // unit visits: the tiles some query block of its rows may attend to (block-masked launches
@@ -407,7 +443,7 @@ __device__ __forceinline__ void tile_list_builder(const AttnParams& p, const Sch
 }
 
 // ---------------------------------------------------------------------------------------
-// TMA producer (one thread).
+// TMA producer (one warp; an elected thread issues the copies).
 // ---------------------------------------------------------------------------------------
 template <int D, bool MASKED>
 __device__ __forceinline__ void producer(const CUtensorMap* tmQ, const CUtensorMap* tmQ128,
@@ -418,6 +454,10 @@ __device__ __forceinline__ void producer(const CUtensorMap* tmQ, const CUtensorM
   using C = Cfg<D>;
   auto bar = [&](int i) { return bar0 + 8u * i; };
   const int nw = (p.nkv + 31) >> 5;
+  const bool lead = elect_one();
+  auto wait = [&](uint32_t b, uint32_t parity) -> bool {
+    return __all_sync(0xffffffffu, mbar_wait(b, parity, abort, kWaitLimitNs));
+  };
   int q_cnt[2] = {0, 0};
   int it = 0;
   // L2 priorities: a query tile is read once, a head's K/V by every unit of that head.  Marking
@@ -430,8 +470,8 @@ __device__ __forceinline__ void producer(const CUtensorMap* tmQ, const CUtensorM
     int w;
     const uint32_t* tw = nullptr;
     if constexpr (MASKED) {
-      if (!mbar_wait(tl.full(k), tl.parity(k), abort, kWaitLimitNs)) {
-        flag_error(p, 0);
+      if (!wait(tl.full(k), tl.parity(k))) {
+        if (lead) flag_error(p, 0);
         goto drain;
       }
       w = tl.unit(k);
@@ -445,11 +485,10 @@ __device__ __forceinline__ void producer(const CUtensorMap* tmQ, const CUtensorM
     for (int X = 0; X < 2; ++X) {
       const int t = 2 * u.pr + X;
       if (t >= sc.tiles) break;
-      if (!mbar_wait(bar(C::kBarQEmpty + X), (q_cnt[X] & 1) ^ 1, abort, kWaitLimitNs)) {
-        flag_error(p, 0);
+      if (!wait(bar(C::kBarQEmpty + X), (q_cnt[X] & 1) ^ 1)) {
+        if (lead) flag_error(p, 0);
         goto drain;
       }
-      mbar_arrive_expect_tx(bar(C::kBarQFull + X), C::kTileBytes);
       const uint32_t dst = sQ0 + X * C::kTileBytes;
       const int r0 = t * BM;
       const int a0 = r0 / p.Np;
@@ -458,27 +497,36 @@ __device__ __forceinline__ void producer(const CUtensorMap* tmQ, const CUtensorM
         // the active list read the following tokens, or zeros past the sequence; they are
         // never stored)
         const int tok = p.active[a0] * p.N + (r0 - a0 * p.Np);
-#pragma unroll
-        for (int hb = 0; hb < C::kHalves; ++hb)
-          tma_load_3d_hint(dst + hb * C::kHalfBytes, tmQ128, bar(C::kBarQFull + X), hb * 64,
-                           u.h, tok, pol_q);
-      } else {
-        // a tile across frames: gathered in boxes of 8 rows (frames are padded to 8 rows)
-        int tok[BM / 8];
-#pragma unroll
-        for (int b = 0; b < BM / 8; ++b) {
-          const int r = r0 + b * 8;
-          const int a = r / p.Np;
-          tok[b] = r < sc.R ? p.active[a] * p.N + (r - a * p.Np)
-                            : p.S_tok;  // past the active list: out of bounds, zero filled
-        }
-#pragma unroll
-        for (int b = 0; b < BM / 8; ++b)
+        if (lead) {
+          mbar_arrive_expect_tx(bar(C::kBarQFull + X), C::kTileBytes);
 #pragma unroll
           for (int hb = 0; hb < C::kHalves; ++hb)
-            tma_load_3d_hint(dst + hb * C::kHalfBytes + b * 1024, tmQ, bar(C::kBarQFull + X),
-                             hb * 64, u.h, tok[b], pol_q);
+            tma_load_3d_hint(dst + hb * C::kHalfBytes, tmQ128, bar(C::kBarQFull + X), hb * 64,
+                             u.h, tok, pol_q);
+        }
+      } else {
+        // a tile across frames: gathered in boxes of 8 rows (frames are padded to 8 rows)
+        // lane b finds the first token of box b
+        int tok = 0;
+        if (const int r = r0 + (threadIdx.x & 31) * 8; (threadIdx.x & 31) < BM / 8) {
+          const int a = r / p.Np;
+          tok = r < sc.R ? p.active[a] * p.N + (r - a * p.Np)
+                         : p.S_tok;  // past the active list: out of bounds, zero filled
+        }
+        if (lead) mbar_arrive_expect_tx(bar(C::kBarQFull + X), C::kTileBytes);
+#pragma unroll 4
+        for (int b = 0; b < BM / 8; ++b) {
+          const int tb = __shfl_sync(0xffffffffu, tok, b);
+          if (lead) {
+#pragma unroll
+            for (int hb = 0; hb < C::kHalves; ++hb)
+              tma_load_3d_hint(dst + hb * C::kHalfBytes + b * 1024, tmQ, bar(C::kBarQFull + X),
+                               hb * 64, u.h, tb, pol_q);
+          }
+          __syncwarp();
+        }
       }
+      __syncwarp();
       ++q_cnt[X];
     }
     // (MASKED, work queue) tiles of this unit still to load; the claim signal goes out once
@@ -488,7 +536,7 @@ __device__ __forceinline__ void producer(const CUtensorMap* tmQ, const CUtensorM
       left = static_cast<int>(tw[kTLWords]);
       claim_due = claim_jit(p, sc);
       if (claim_due && left <= kClaimAhead) {
-        mbar_arrive(tl.claim());
+        if (lead) mbar_arrive(tl.claim());
         claim_due = false;
       }
     }
@@ -497,27 +545,30 @@ __device__ __forceinline__ void producer(const CUtensorMap* tmQ, const CUtensorM
          j = tile_next<MASKED>(tw, nw, j)) {
       if constexpr (MASKED) {
         if (claim_due && --left <= kClaimAhead) {
-          mbar_arrive(tl.claim());
+          if (lead) mbar_arrive(tl.claim());
           claim_due = false;
         }
       }
 #pragma unroll
       for (int kv = 0; kv < 2; ++kv) {
         const int s = it % C::kSlots, n = it / C::kSlots;
-        if (!mbar_wait(bar(C::kBarKVEmpty + s), (n & 1) ^ 1, abort, kWaitLimitNs)) {
-          flag_error(p, 1);
+        if (!wait(bar(C::kBarKVEmpty + s), (n & 1) ^ 1)) {
+          if (lead) flag_error(p, 1);
           goto drain;
         }
-        mbar_arrive_expect_tx(bar(C::kBarKVFull + s), C::kTileBytes);
-        const uint32_t dst = sKV0 + s * C::kTileBytes;
+        if (lead) {
+          mbar_arrive_expect_tx(bar(C::kBarKVFull + s), C::kTileBytes);
+          const uint32_t dst = sKV0 + s * C::kTileBytes;
 #pragma unroll
-        for (int hb = 0; hb < C::kHalves; ++hb)
-          tma_load_3d_hint(dst + hb * C::kHalfBytes, kv ? tmV : tmK, bar(C::kBarKVFull + s),
-                           hb * 64, u.h, j * BN, pol_kv);
+          for (int hb = 0; hb < C::kHalves; ++hb)
+            tma_load_3d_hint(dst + hb * C::kHalfBytes, kv ? tmV : tmK, bar(C::kBarKVFull + s),
+                             hb * 64, u.h, j * BN, pol_kv);
+        }
+        __syncwarp();
         ++it;
       }
     }
-    if constexpr (MASKED) mbar_arrive(tl.empty(k));
+    if constexpr (MASKED) warp_arrive(tl.empty(k));
   }
 drain:
   // every armed fill has all its copies issued; wait for the last fill of each buffer
@@ -528,143 +579,154 @@ drain:
 }
 
 // ---------------------------------------------------------------------------------------
-// MMA issuer (one thread).
+// MMA issuer of query tile X (one warp; an elected thread issues the MMAs).
 // ---------------------------------------------------------------------------------------
 // Descriptors are built once per buffer; a K step only adds its byte offset / 16 to the start
-// address field (bits 0-13), which cannot carry: every shared address is below 256 KB.  (The
-// single issuing thread is on the critical path: rebuilding descriptors per MMA cost ~2-4%.)
-template <int D>
+// address field (bits 0-13), which cannot carry: every shared address is below 256 KB.
+// S = Q K^T over the columns [16 K0, 16 K1) of the head dim.
+template <int D, int K0, int K1>
 __device__ __forceinline__ void mma_qk(uint32_t tS, uint64_t dQ, uint64_t dK) {
   constexpr uint32_t idesc = idesc_bf16_f32(BM, BN, 0, 0);
 #pragma unroll
-  for (int k = 0; k < D / 16; ++k) {
+  for (int k = K0; k < K1; ++k) {
     const uint64_t off = ((k >> 2) * (BM * 128) + (k & 3) * 32) >> 4;
     tc_mma_ss(tS, dQ + off, dK + off, idesc, k > 0);
   }
 }
 
-template <int D>
+// O (+)= P V over the keys [16 K0, 16 K1) of the tile.
+template <int D, int K0, int K1>
 __device__ __forceinline__ void mma_pv(uint32_t tO, uint32_t tP, uint64_t dV, uint32_t acc) {
   constexpr uint32_t idesc = idesc_bf16_f32(BM, D, 0, 1);
 #pragma unroll
-  for (int k = 0; k < BN / 16; ++k)
+  for (int k = K0; k < K1; ++k)
     tc_mma_ts(tO, tP + k * 8, dV + ((k * 2048) >> 4), idesc, (acc | k) != 0);
 }
 
 template <int D, bool MASKED>
-__device__ __forceinline__ void mma_issuer(const AttnParams& p, const Sched& sc, uint32_t tmem,
-                                           uint32_t sQ0, uint32_t sKV0, uint32_t bar0,
-                                           const TLRing& tl, volatile int* abort) {
+__device__ __forceinline__ bool mma_issuer(const AttnParams& p, const Sched& sc, int X,
+                                           uint32_t tmem, uint32_t sQ0, uint32_t sKV0,
+                                           uint32_t bar0, const TLRing& tl, volatile int* abort) {
   using C = Cfg<D>;
+  constexpr int kEarly = D / 16 - kTurnAhead<D>;
+  const bool lead = elect_one();
   auto bar = [&](int i) { return bar0 + 8u * i; };
-  const uint32_t tS[2] = {tmem, tmem + 128};
-  const uint32_t tO[2] = {tmem + 256, tmem + 384};
-  const uint64_t dQ[2] = {smem_desc_sw128(sQ0, 16, 1024),
-                          smem_desc_sw128(sQ0 + C::kTileBytes, 16, 1024)};
+  const uint32_t tS = tmem + X * 128, tO = tmem + 256 + X * 128;
+  const uint64_t dQ = smem_desc_sw128(sQ0 + X * C::kTileBytes, 16, 1024);
   // K operand: K-major; V operand: MN-major with the two 64-column halves 16 KB apart
   auto dK = [&](int s) { return smem_desc_sw128(sKV0 + s * C::kTileBytes, 16, 1024); };
   auto dV = [&](int s) { return smem_desc_sw128(sKV0 + s * C::kTileBytes, BN * 128, 1024); };
-  int q_cnt[2] = {0, 0};
-  int p_cnt[2] = {0, 0};
-  int it = 0;
-  auto next_slot = [&](int& s) -> bool {
-    s = it % C::kSlots;
-    const bool ok = mbar_wait(bar(C::kBarKVFull + s), (it / C::kSlots) & 1, abort, kWaitLimitNs);
-    ++it;
-    tc_fence_after();
-    return ok;
+  int q_cnt = 0, it = 0;
+  bool my_turn = X == 0;  // the first turn is tile A's
+  auto wait = [&](uint32_t b, uint32_t parity) -> bool {
+    return __all_sync(0xffffffffu, mbar_wait(b, parity, abort, kWaitLimitNs));
   };
-  auto wait_p = [&](int X) -> bool {
-    const bool ok = mbar_wait(bar(C::kBarPFull + X), p_cnt[X] & 1, abort, kWaitLimitNs);
-    ++p_cnt[X];
-    tc_fence_after();
-    return ok;
+  auto wait_slot = [&](int i) -> bool {
+    return wait(bar(C::kBarKVFull + i % C::kSlots), (i / C::kSlots) & 1);
+  };
+  auto take_turn = [&]() {
+    if (!my_turn) named_sync(turn_barrier(X), 64);
+    my_turn = false;
   };
   for (int k = 0;; ++k) {  // k: units so far (MASKED: tile-list ring position)
     int w;
     const uint32_t* tw = nullptr;
     if constexpr (MASKED) {
-      if (!mbar_wait(tl.full(k), tl.parity(k), abort, kWaitLimitNs)) goto fail;
+      if (!wait(tl.full(k), tl.parity(k))) break;
       w = tl.unit(k);
-      if (w < 0) break;
+      if (w < 0) return true;
       tw = tl.words(k);
     } else {
       w = blockIdx.x + k * static_cast<int>(gridDim.x);
-      if (w >= sc.units) break;
+      if (w >= sc.units) return true;
     }
     const Unit u = get_unit(sc, p, w);
     const bool hasB = 2 * u.pr + 1 < sc.tiles;
     // number of KV tiles of the unit: j1 - j0, or (MASKED) the set bits of the builder's
     // bitmap (the issuer needs only the count; the producer walks the bits)
     const int ntiles = MASKED ? static_cast<int>(tw[kTLWords]) : u.j1 - u.j0;
-    if (!mbar_wait(bar(C::kBarQFull + 0), q_cnt[0] & 1, abort, kWaitLimitNs)) goto fail;
-    ++q_cnt[0];
-    if (hasB) {
-      if (!mbar_wait(bar(C::kBarQFull + 1), q_cnt[1] & 1, abort, kWaitLimitNs)) goto fail;
-      ++q_cnt[1];
+    if (X == 1 && !hasB) {
+      // no second query tile: only give the K/V slots back
+      bool ok = true;
+      for (int i = 0; ok && i < 2 * ntiles; ++i, ++it) {
+        ok = wait_slot(it);
+        if (ok && lead) mbar_arrive(bar(C::kBarKVEmpty + it % C::kSlots));
+        __syncwarp();
+      }
+      if (!ok) break;
+      if constexpr (MASKED) warp_arrive(tl.empty(k));
+      continue;
     }
+    if (!wait(bar(C::kBarQFull + X), q_cnt & 1)) break;
+    ++q_cnt;
     tc_fence_after();
     if (MASKED && ntiles == 0) {
       // no allowed key block: release the queries.  No output barrier is committed: the
       // softmax warps see the same empty tile list and write their result without waiting
       // (a commit here could run two phases ahead of them).
-      mbar_arrive(tl.empty(k));
-      tc_commit(bar(C::kBarQEmpty + 0));
-      if (hasB) tc_commit(bar(C::kBarQEmpty + 1));
+      warp_arrive(tl.empty(k));
+      if (lead) tc_commit(bar(C::kBarQEmpty + X));
+      __syncwarp();
       continue;
     }
-    int sK, sV;
-    if (!next_slot(sK)) goto fail;
-    mma_qk<D>(tS[0], dQ[0], dK(sK));
-    tc_commit(bar(C::kBarSFull + 0));
-    if (hasB) {
-      mma_qk<D>(tS[1], dQ[1], dK(sK));
-      tc_commit(bar(C::kBarSFull + 1));
+    if (!wait_slot(it) || !__all_sync(0xffffffffu, *abort == 0)) break;
+    if (hasB) take_turn();
+    if (lead) mma_qk<D, 0, kEarly>(tS, dQ, dK(it % C::kSlots));
+    __syncwarp();
+    if (hasB) named_arrive(turn_barrier(X ^ 1), 64);
+    if (lead) {
+      mma_qk<D, kEarly, D / 16>(tS, dQ, dK(it % C::kSlots));
+      tc_commit(bar(C::kBarSFull + X));
+      tc_commit(bar(C::kBarKVEmpty + it % C::kSlots));
     }
-    tc_commit(bar(C::kBarKVEmpty + sK));
-    if (!next_slot(sV)) goto fail;
-    if (!wait_p(0)) goto fail;
-    mma_pv<D>(tO[0], tS[0], dV(sV), 0);
-    int nj = 1;  // tiles issued so far
+    __syncwarp();
+    ++it;
+    bool ok = true;
 #pragma unroll 1
-    for (int j = 0;; ++j) {
-      if (j + 1 >= ntiles) break;
-      ++nj;
-      if (!next_slot(sK)) goto fail;
-      mma_qk<D>(tS[0], dQ[0], dK(sK));
-      tc_commit(bar(C::kBarSFull + 0));
-      if (hasB) {
-        if (!wait_p(1)) goto fail;
-        mma_pv<D>(tO[1], tS[1], dV(sV), j > 0);
+    for (int j = 0; j < ntiles; ++j) {
+      const bool more = j + 1 < ntiles;
+      const int sV = it % C::kSlots, sK = (it + 1) % C::kSlots;
+      // V(j) and K(j+1), waited for while the other tile's MMAs run
+      ok = wait_slot(it) && (!more || wait_slot(it + 1));
+      it += more ? 2 : 1;
+      ok = ok && *abort == 0;
+      if (!__all_sync(0xffffffffu, ok)) break;
+      if (hasB) take_turn();
+      named_sync(p_barrier(X, 0), kPThreads);
+      tc_fence_after();
+      if (lead) mma_pv<D, 0, kPSplit / 16>(tO, tS, dV(sV), j > 0);
+      __syncwarp();
+      if (kPSplit < BN) {
+        named_sync(p_barrier(X, 1), kPThreads);
+        tc_fence_after();
       }
-      tc_commit(bar(C::kBarKVEmpty + sV));
-      if (hasB) {
-        mma_qk<D>(tS[1], dQ[1], dK(sK));
-        tc_commit(bar(C::kBarSFull + 1));
+      if (lead) {
+        mma_pv<D, kPSplit / 16, BN / 16>(tO, tS, dV(sV), 1);
+        if (more) mma_qk<D, 0, kEarly>(tS, dQ, dK(sK));
       }
-      tc_commit(bar(C::kBarKVEmpty + sK));
-      if (!next_slot(sV)) goto fail;
-      if (!wait_p(0)) goto fail;
-      mma_pv<D>(tO[0], tS[0], dV(sV), 1);
+      __syncwarp();
+      if (hasB) named_arrive(turn_barrier(X ^ 1), 64);
+      if (lead) {
+        if (more) {
+          mma_qk<D, kEarly, D / 16>(tS, dQ, dK(sK));
+          tc_commit(bar(C::kBarSFull + X));
+          // the unit's last QK^T: the next unit's queries may load during the last softmax and PV
+          if (j + 2 == ntiles) tc_commit(bar(C::kBarQEmpty + X));
+          tc_commit(bar(C::kBarKVEmpty + sV));
+          tc_commit(bar(C::kBarKVEmpty + sK));
+        } else {
+          tc_commit(bar(C::kBarODone + X));
+          if (ntiles == 1) tc_commit(bar(C::kBarQEmpty + X));
+          tc_commit(bar(C::kBarKVEmpty + sV));
+        }
+      }
+      __syncwarp();
     }
-    if constexpr (MASKED) mbar_arrive(tl.empty(k));
-    tc_commit(bar(C::kBarODone + 0));
-    tc_commit(bar(C::kBarQEmpty + 0));
-    if (hasB) {
-      if (!wait_p(1)) goto fail;
-      mma_pv<D>(tO[1], tS[1], dV(sV), nj > 1);
-      tc_commit(bar(C::kBarODone + 1));
-      tc_commit(bar(C::kBarQEmpty + 1));
-    }
-    tc_commit(bar(C::kBarKVEmpty + sV));
+    if (!ok) break;
+    if constexpr (MASKED) warp_arrive(tl.empty(k));
   }
-  goto drain;
-fail:
-  flag_error(p, 2);
-drain:
-  // all MMAs issued so far complete before TMEM is released
-  tc_commit(bar(C::kBarDrain));
-  drain_wait(bar(C::kBarDrain), 0);
+  if (lead) flag_error(p, 2);
+  return false;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -685,7 +747,7 @@ __device__ __forceinline__ void store_row_bf16(uint16_t* orow, const float* o, f
 }
 
 template <int D, bool MASKED>
-__device__ __forceinline__ void softmax_group(const AttnParams& p, const Sched& sc, int X,
+__device__ __forceinline__ bool softmax_group(const AttnParams& p, const Sched& sc, int X,
                                               uint32_t tmem, uint32_t bar0, const TLRing& tl,
                                               volatile int* abort, volatile int* merge_flag) {
   using C = Cfg<D>;
@@ -707,7 +769,7 @@ __device__ __forceinline__ void softmax_group(const AttnParams& p, const Sched& 
       // slot's release count is the same for all units
       if (!__all_sync(0xffffffffu, mbar_wait(tl.full(k), tl.parity(k), abort, kWaitLimitNs))) {
         flag_error(p, 8);
-        return;
+        return false;
       }
       w = tl.unit(k);
       if (w < 0) break;
@@ -752,7 +814,7 @@ __device__ __forceinline__ void softmax_group(const AttnParams& p, const Sched& 
       if (!__all_sync(0xffffffffu, mbar_wait(bar(C::kBarSFull + X), s_cnt & 1, abort,
                                             kWaitLimitNs))) {
         flag_error(p, 3);
-        return;
+        return false;
       }
       ++s_cnt;
       tc_fence_after();
@@ -790,34 +852,6 @@ __device__ __forceinline__ void softmax_group(const AttnParams& p, const Sched& 
         l *= fac;
         m = m_new;
       }
-      // p = 2^(s*scale*log2(e) - m) with packed fp32 pairs for the scale/subtract and the
-      // row sum (8 independent sum chains in 4 packed accumulators)
-      // (MASKED) while every key seen so far was excluded, m is -inf: use 0 so p = 2^-inf = 0;
-      // for a tile the row may not see, an offset of -inf gives p = 0 for every key (s is
-      // finite or -inf, so s * scale - inf is -inf, never NaN)
-      const float nm = (MASKED && mk == 0u) ? -INFINITY : (MASKED && m == -INFINITY) ? 0.f : -m;
-      const uint64_t sl2x2 = f2_pack(sl2, sl2), nmx2 = f2_pack(nm, nm);
-      uint64_t l4[4] = {0ull, 0ull, 0ull, 0ull};
-#pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        uint32_t pk[32];
-#pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          float x0, x1;
-          f2_unpack(ffma2(f2_pack(sf[half * 64 + 2 * e], sf[half * 64 + 2 * e + 1]), sl2x2, nmx2),
-                    x0, x1);
-          const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
-          l4[e & 3] = fadd2(l4[e & 3], f2_pack(p0, p1));
-          pk[e] = pack_bf16x2(p0, p1);
-        }
-        tmem_st32(tS + half * 32, pk);
-      }
-      {
-        const uint64_t t2 = fadd2(fadd2(l4[0], l4[1]), fadd2(l4[2], l4[3]));
-        float a, b;
-        f2_unpack(t2, a, b);
-        l += a + b;
-      }
       // O was last written by the previous tile's PV, which completed before S(j) was
       // signalled; at the unit's first tile it holds nothing yet
       if (rescale && (MASKED ? !first : j > u.j0)) {
@@ -831,9 +865,39 @@ __device__ __forceinline__ void softmax_group(const AttnParams& p, const Sched& 
           tmem_st32(tO + c * 32, o);
         }
       }
-      tmem_wait_st();
-      tc_fence_before();
-      mbar_arrive(bar(C::kBarPFull + X));
+      // p = 2^(s*scale*log2(e) - m) with packed fp32 pairs for the scale/subtract and the
+      // row sum (8 independent sum chains in 4 packed accumulators)
+      // (MASKED) while every key seen so far was excluded, m is -inf: use 0 so p = 2^-inf = 0;
+      // for a tile the row may not see, an offset of -inf gives p = 0 for every key (s is
+      // finite or -inf, so s * scale - inf is -inf, never NaN)
+      const float nm = (MASKED && mk == 0u) ? -INFINITY : (MASKED && m == -INFINITY) ? 0.f : -m;
+      const uint64_t sl2x2 = f2_pack(sl2, sl2), nmx2 = f2_pack(nm, nm);
+      uint64_t l4[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        uint32_t pk[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          float x0, x1;
+          f2_unpack(ffma2(f2_pack(sf[q * 32 + 2 * e], sf[q * 32 + 2 * e + 1]), sl2x2, nmx2),
+                    x0, x1);
+          const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
+          l4[e & 3] = fadd2(l4[e & 3], f2_pack(p0, p1));
+          pk[e] = pack_bf16x2(p0, p1);
+        }
+        tmem_st16(tS + q * 16, pk);
+        if ((q + 1) * 32 == kPSplit || (q == 3 && kPSplit < BN)) {
+          tmem_wait_st();
+          tc_fence_before();
+          named_arrive(p_barrier(X, q == 3 && kPSplit < BN), kPThreads);
+        }
+      }
+      {
+        const uint64_t t2 = fadd2(fadd2(l4[0], l4[1]), fadd2(l4[2], l4[3]));
+        float a, b;
+        f2_unpack(t2, a, b);
+        l += a + b;
+      }
       first = false;
       j = jn;
       mk = mk_next;
@@ -844,7 +908,7 @@ __device__ __forceinline__ void softmax_group(const AttnParams& p, const Sched& 
       if (!__all_sync(0xffffffffu,
                       mbar_wait(bar(C::kBarODone + X), o_cnt & 1, abort, kWaitLimitNs))) {
         flag_error(p, 4);
-        return;
+        return false;
       }
       ++o_cnt;
       tc_fence_after();
@@ -903,7 +967,7 @@ __device__ __forceinline__ void softmax_group(const AttnParams& p, const Sched& 
     ++split_cnt;
     if (!group_sync(bar(C::kBarGroup + X), g_cnt, abort)) {  // every row is published
       flag_error(p, 5);
-      return;
+      return false;
     }
     if (row == 0) {
       const int old = atomicAdd(p.ws_count + 2 * u.item + X, 1);
@@ -911,7 +975,7 @@ __device__ __forceinline__ void softmax_group(const AttnParams& p, const Sched& 
     }
     if (!group_sync(bar(C::kBarGroup + X), g_cnt, abort)) {  // the flag is visible
       flag_error(p, 6);
-      return;
+      return false;
     }
     if (*flag == 0) continue;
     __threadfence();
@@ -954,6 +1018,18 @@ __device__ __forceinline__ void softmax_group(const AttnParams& p, const Sched& 
     }
     if (row == 0) p.ws_count[2 * u.item + X] = 0;  // ready for the next launch
   }
+  return true;
+}
+
+// A warp that gives up: release the MMA warp that waits for it until that warp has left (2 s at
+// most: it reads the abort flag, which is up, in every round).
+__device__ __forceinline__ void release_mma(const volatile int* done, int bar_a, int bar_b,
+                                            int threads) {
+  for (int n = 0; n < 2000000 && !__all_sync(0xffffffffu, *done != 0); ++n) {
+    named_arrive(bar_a, threads);
+    if (bar_b != bar_a) named_arrive(bar_b, threads);
+    __nanosleep(1000);
+  }
 }
 
 template <int D, bool MASKED>
@@ -971,24 +1047,25 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
   volatile int* abort = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
   volatile int* merge_flag = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 8);  // [2][2]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  volatile int* mma_done = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 24);  // [2]
+  const int warp = threadIdx.x >> 5;
 
   if (threadIdx.x == 0) {
     for (int X = 0; X < 2; ++X) {
       mbar_init(bar0 + 8 * (C::kBarQFull + X), 1);
       mbar_init(bar0 + 8 * (C::kBarQEmpty + X), 1);
       mbar_init(bar0 + 8 * (C::kBarSFull + X), 1);
-      mbar_init(bar0 + 8 * (C::kBarPFull + X), 128);
       mbar_init(bar0 + 8 * (C::kBarODone + X), 1);
+      mbar_init(bar0 + 8 * (C::kBarDrain + X), 1);
       mbar_init(bar0 + 8 * (C::kBarGroup + X), 128);
       merge_flag[2 * X] = 0;
       merge_flag[2 * X + 1] = 0;
+      mma_done[X] = 0;
     }
     for (int s = 0; s < C::kSlots; ++s) {
       mbar_init(bar0 + 8 * (C::kBarKVFull + s), 1);
-      mbar_init(bar0 + 8 * (C::kBarKVEmpty + s), 1);
+      mbar_init(bar0 + 8 * (C::kBarKVEmpty + s), 2);
     }
-    mbar_init(bar0 + 8 * C::kBarDrain, 1);
     if constexpr (MASKED) {
       for (int s = 0; s < kTLSlots; ++s) {
         mbar_init(sbase + C::kOffTL + 8 * s, 32);
@@ -1021,18 +1098,25 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp < 4) {
     reg_dealloc<kRegsControl>();
     if (warp == 0) {
-      if (lane == 0) producer<D, MASKED>(&tmQ, &tmQ128, &tmK, &tmV, p, sc, sQ0, sKV0, bar0, tl, abort);
+      producer<D, MASKED>(&tmQ, &tmQ128, &tmK, &tmV, p, sc, sQ0, sKV0, bar0, tl, abort);
+    } else if (warp < 3) {
+      const int X = warp - 1;
+      const bool ok = mma_issuer<D, MASKED>(p, sc, X, tmem, sQ0, sKV0, bar0, tl, abort);
       __syncwarp();
-    } else if (warp == 1) {
-      if (lane == 0) mma_issuer<D, MASKED>(p, sc, tmem, sQ0, sKV0, bar0, tl, abort);
+      mma_done[X] = 1;  // waits on no named barrier any more
+      if (!ok) release_mma(mma_done + (X ^ 1), turn_barrier(X ^ 1), turn_barrier(X ^ 1), 64);
+      // all MMAs issued so far complete before TMEM is released
+      if (elect_one()) tc_commit(bar0 + 8 * (C::kBarDrain + X));
       __syncwarp();
-    } else if (MASKED && warp == 2) {
+      drain_wait(bar0 + 8 * (C::kBarDrain + X), 0);
+    } else if (MASKED) {
       tile_list_builder(p, sc, tl, abort);
     }
   } else {
     reg_alloc<kRegsSoftmax>();
     const int X = (warp - 4) >> 2;
-    softmax_group<D, MASKED>(p, sc, X, tmem, bar0, tl, abort, merge_flag + 2 * X);
+    if (!softmax_group<D, MASKED>(p, sc, X, tmem, bar0, tl, abort, merge_flag + 2 * X))
+      release_mma(mma_done + X, p_barrier(X, 0), p_barrier(X, 1), kPThreads);
   }
 
   tc_fence_before();

@@ -17,6 +17,13 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
   return t;
 }
 
+// Low half of the same timer: wraps every 4.29 s, enough for the limits of the waits.
+__device__ __forceinline__ uint32_t globaltimer_lo_ns() {
+  uint32_t t;
+  asm volatile("mov.u32 %0, %%globaltimer_lo;" : "=r"(t));
+  return t;
+}
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
@@ -43,26 +50,49 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
+// The same without waiting: has the phase completed?
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // Wait until the phase with the given parity of barrier `bar` has completed.
 // Gives up after `limit_ns` of wall-clock time or as soon as another thread of the CTA has
 // raised *abort; on expiry it raises *abort itself.  Returns false when it gave up.  A spin
-// count (limit_ns / 16 rounds of 32 polls, far more than the time limit allows) bounds the
-// loop even if the timer did not advance.
+// count (limit_ns polls, far more than the time limit allows) bounds the
+// loop even if the timer did not advance.  The timer is first read after 32 polls: reading it
+// earlier put 60-90 cycles on a hand-off of two warps (a ping-pong of 511 cycles, 422 without).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort,
-                                          uint64_t limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer_ns();
-  const uint64_t max_rounds = limit_ns >> 4;
-  for (uint64_t n = 0;; ++n) {
+                                          uint32_t limit_ns) {
+  uint32_t t0 = 0;
 #pragma unroll 1
-    for (int i = 0; i < 32; ++i)
-      if (mbar_try_wait(bar, parity)) return true;
+  for (uint32_t n = 0;; ++n) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((n & 31) != 31) continue;
     if (*abort) return false;
-    if (n >= max_rounds || globaltimer_ns() - t0 > limit_ns) {
+    const uint32_t t = globaltimer_lo_ns();
+    if (n == 31) t0 = t;
+    if (n >= limit_ns || t - t0 > limit_ns) {
       *abort = 1;
       return false;
     }
   }
+}
+
+// ---------------------------------------------------------------- named barriers
+// Warps arrive on hardware barrier `id`; `threads` counts the arriving and the waiting ones.
+__device__ __forceinline__ void named_arrive(int id, int threads) {
+  asm volatile("barrier.cta.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void named_sync(int id, int threads) {
+  asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
 // ---------------------------------------------------------------- TMA
@@ -110,6 +140,20 @@ __device__ __forceinline__ void tc_fence_before() {
 }
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+// One thread of the converged warp (nonzero in that thread).  tcgen05 and bulk-copy instructions
+// take their operands from uniform registers: under a branch on elect.sync the compiler knows
+// that one thread runs them and issues each at once; under a branch on the lane number it does
+// not, and 16 MMAs and a commit took 1098 cycles to issue whatever their size (390 this way, at
+// N = 16).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok));
+  return ok != 0;
 }
 // Arrive once on `bar` when every tcgen05 async op issued so far by this thread is done.
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
