@@ -819,6 +819,26 @@ def test_frame_gram_matches_fp64_matmul(cuda_lib, F, E, ld):
     assert err.max() < 1e-5, err.max()
 
 
+@pytest.mark.parametrize("F", [1, 8, 9, 16, 17, 40, 41, 48, 64])
+@pytest.mark.parametrize("E,pad,shift", [(1, 0, 0), (127, 1, 0), (129, 3, 1), (3071, 1, 0),
+                                         (57600 + 5, 3, 0), (117000, 0, 1)])
+def test_frame_gram_tile_and_slice_edges(cuda_lib, F, E, pad, shift):
+    """Frame groups of 8, slices cut short, rows and bases off the 16-byte boundaries.  Each fp32
+    chain has at most 512 products (a CTA's elements over its k-groups), the rest is summed
+    without loss, so |error| <= 512 * 2^-24 * sum |p_i p_j|."""
+    rf = cuda_lib
+    g = torch.Generator(device=DEV).manual_seed(F * 7 + E)
+    buf = torch.randn(F * (E + pad) + shift, generator=g, device=DEV)
+    P = buf[shift:].view(F, E + pad)[:, :E]
+    G = torch.full((F, F), 9.0, dtype=torch.float64, device=DEV)
+    rf.rf_frame_gram(P, G)
+    torch.cuda.synchronize()
+    p = P.double()
+    bound = 512 * 2.0 ** -24 * (p.abs() @ p.abs().t())
+    assert ((G - p @ p.t()).abs() <= bound).all()
+    assert torch.equal(G, G.t())
+
+
 def test_keyframes_from_device_gram_match_oracle(cuda_lib):
     """Scene-structured proxies (5 scenes over 21 frames of 3600 tokens x 16 channels):
     the keyframes are the scene starts, as the oracle's Algorithm 1 finds them."""
