@@ -19,11 +19,12 @@ planner rf_plan_build and is uploaded once.  PyTorch only allocates memory.
 from __future__ import annotations
 
 from dataclasses import dataclass
+from operator import index
 from typing import Optional
 
 import torch
 
-from . import (rf_attn, rf_attn_workspace_bytes, rf_pipeline_bytes, rf_pipeline_create,
+from . import (_stream, rf_attn, rf_attn_workspace_bytes, rf_pipeline_bytes, rf_pipeline_create,
                rf_pipeline_destroy, rf_pipeline_step, rf_pipeline_sync, rf_plan_build, rf_project,
                rf_project_kv, rf_schedule_compact, rf_step)
 
@@ -42,6 +43,15 @@ def upload_plan(F, S, is_key, stride, T_w, device, sigma=None) -> Plan:
     h = rf_plan_build(F, S, is_key, stride, T_w, sigma)
     t = {k: torch.from_numpy(v).to(device) for k, v in h.items()}
     return Plan(t["mask"], t["alpha"], t["beta"], t["dt"], t["cur_slot"], h)
+
+
+def _row(t: torch.Tensor, s: int) -> int:
+    """Device address of t[s] for a [S, F] plan tensor, without making the view (2 us of host
+    time each, eight per step; a step of 4 x 64 tokens is bound by the host)."""
+    s, S = index(s), t.shape[0]
+    if not -S <= s < S:
+        raise IndexError(f"step {s} is out of range for a plan of {S} steps")
+    return t.data_ptr() + (s % S) * t.stride(0) * t.element_size()
 
 
 class StepCore:
@@ -97,29 +107,30 @@ class StepCore:
         return self.z2[slot, idx]
 
     def compact(self, s: int, stream=None):
-        rf_schedule_compact(self.plan.mask[s], self.F, self.N, self.active, self.skipped,
+        rf_schedule_compact(_row(self.plan.mask, s), self.F, self.N, self.active, self.skipped,
                             self.token_idx, self.counts, stream)
 
     def project(self, s: int, stream=None):
-        rf_project(self.ctx, self.z2, self.plan.cur_slot[s], self.plan.alpha[s],
-                   self.plan.beta[s], self.F, self.E, stream)
+        rf_project(self.ctx, self.z2, _row(self.plan.cur_slot, s), _row(self.plan.alpha, s),
+                   _row(self.plan.beta, s), self.F, self.E, stream)
 
     def project_kv(self, s: int, K, V, stream=None):
-        rf_project_kv(K, V, K.stride(0), self.Kc, self.Vc, self.plan.cur_slot[s],
-                      self.plan.alpha[s], self.plan.beta[s], self.active, self.skipped,
-                      self.counts, self.F, self.N, self.H * self.d, stream)
+        rf_project_kv(K, V, K.stride(0), self.Kc, self.Vc, _row(self.plan.cur_slot, s),
+                      _row(self.plan.alpha, s), _row(self.plan.beta, s), self.active,
+                      self.skipped, self.counts, self.F, self.N, self.H * self.d, stream)
 
     def attn(self, O, Q, K, V, scale: float, lse: Optional[torch.Tensor] = None, stream=None):
         rf_attn(O, lse, Q, K, V, Q.stride(0), O.stride(0), self.F, self.N, self.H, self.d,
                 self.active, self.counts, scale, self.workspace, self.status, stream)
 
     def step(self, s: int, v: torch.Tensor, stream=None):
-        rf_step(self.z2, self.plan.cur_slot[s], v, self.plan.dt[s], self.active, self.counts,
-                self.F, self.E, stream)
+        rf_step(self.z2, _row(self.plan.cur_slot, s), v, _row(self.plan.dt, s), self.active,
+                self.counts, self.F, self.E, stream)
 
     def run(self, s: int, v, O, Q, K, V, scale: float, lse=None, stream=None):
         """Step s.  Q, K, V hold the active frames' fresh rows; with the cache, the skipped
         frames' rows of K and V are overwritten with their projection before the attention."""
+        stream = _stream(stream)  # looked up once for the five calls
         self.compact(s, stream)
         self.project(s, stream)
         if self.Kc is not None:

@@ -246,3 +246,19 @@ def test_bench_traffic_figures_belong_to_the_current_kernel():
     for name, entry in bench.ATTN_TRAFFIC.items():
         assert entry["code_sha256_rf_attn_cu"] == sha, name
         assert entry["bytes_per_launch"] > 0
+
+
+def test_plan_row_addresses():
+    """stepcore._row is t[s].data_ptr() without the view: every step, negative steps, strided
+    plans, and the same error past the ends."""
+    import torch
+
+    from paper_2606_06309_gb300.stepcore import _row
+    for t in (torch.zeros(7, 5, dtype=torch.uint8), torch.zeros(7, 5),
+              torch.zeros(9, 12)[1:8, 3:8], torch.zeros(14, 5)[::2]):
+        for s in range(-7, 7):
+            assert _row(t, s) == t[s].data_ptr(), s
+        assert _row(t, np.int64(3)) == t[3].data_ptr()
+        for s in (7, -8):
+            with pytest.raises(IndexError):
+                _row(t, s)
