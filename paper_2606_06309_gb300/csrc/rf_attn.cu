@@ -96,6 +96,11 @@ constexpr uint32_t kWaitLimitNs = 2000000000u;  // 2 s: no legitimate wait comes
 constexpr uint64_t kDrainLimitNs = 200000000ull;  // 0.2 s for in-flight copies at teardown
 constexpr float kRescaleLog2 = 8.0f;
 constexpr int kMaxSplit = 16;          // KV ranges per split item
+// KV tiles per range of a split item, at least: a merge costs about as much as the KV steps of
+// that many tiles (us per launch with at least 1, 2, 4, 8 tiles per range:
+// 4 x 64 tokens x 2 heads x 64 12.1, 8.8, 8.8, 8.8; 8 x 200 x 2 x 128 30.9, 26.3, 23.4, 23.7;
+// 5 x 400 x 3 x 64 18.6, 18.6, 17.4, 20.2; 21 x 200 x 3 x 128 37.4, 37.5, 30.8, 29.9).
+constexpr int kMinSplitTiles = 4;
 constexpr int kMaxGrid = 1024;         // workspace is sized for at most this many CTAs
 // Block-masked launches: a ring of per-unit KV-tile bitmaps in shared memory, one bit per KV
 // tile (so at most kTLWords * 32 tiles of 128 keys), followed by the number of set bits.
@@ -182,7 +187,7 @@ __device__ __forceinline__ Sched make_sched(const AttnParams& p) {
     const int tail = T - (rounds - 1) * G;
     int c = G / tail;
     if (c > kMaxSplit) c = kMaxSplit;
-    if (c > p.nkv) c = p.nkv;
+    if (c > p.nkv / kMinSplitTiles) c = p.nkv / kMinSplitTiles;
     if (c >= 2) {
       s.T_full = (rounds - 1) * G;
       s.C = c;
@@ -944,23 +949,25 @@ __device__ __forceinline__ bool softmax_group(const AttnParams& p, const Sched& 
             (MASKED && l == 0.f) ? -INFINITY : (m + __log2f(l)) * 0.69314718055994531f;
       continue;
     }
-    // split item: publish this KV range's partial row, then the last range to finish merges
-    float* part = p.ws_part + ((static_cast<int64_t>(u.part) * 2 + X) * BM + row) * C::kPartFloats;
+    // split item: publish this KV range's partial rows, then the last range to finish merges.  A
+    // tile's partials are [D/4] float4 columns of 128 rows, then {m, l} of the rows: a warp's
+    // stores and loads are 512 consecutive bytes.  (With each row's 528 bytes together and one
+    // range at a time in the merge, 4 x 256 tokens x 2 heads x 128 in 8 ranges took 69 us, now in 2
+    // ranges 17.6; 7 x 1003 x 2 x 128 in 7 ranges 69.6 -> 45.9.)
+    float4* part = reinterpret_cast<float4*>(p.ws_part) +
+                   static_cast<int64_t>(u.part * 2 + X) * (BM * C::kPartFloats / 4) + row;
 #pragma unroll 1
     for (int c = 0; c < D / 32; ++c) {
       uint32_t o[32];
       tmem_ld32(tO + c * 32, o);
       tmem_wait_ld();
-      float4* dst = reinterpret_cast<float4*>(part + c * 32);
-      const bool none = MASKED && l == 0.f;  // no allowed key in this range: O is not written
 #pragma unroll
       for (int q = 0; q < 8; ++q)
-        __stcg(dst + q, none ? make_float4(0.f, 0.f, 0.f, 0.f)
-                             : make_float4(__uint_as_float(o[4 * q]), __uint_as_float(o[4 * q + 1]),
-                                           __uint_as_float(o[4 * q + 2]),
-                                           __uint_as_float(o[4 * q + 3])));
+        __stcg(part + (c * 8 + q) * BM,
+               make_float4(__uint_as_float(o[4 * q]), __uint_as_float(o[4 * q + 1]),
+                           __uint_as_float(o[4 * q + 2]), __uint_as_float(o[4 * q + 3])));
     }
-    __stcg(reinterpret_cast<float4*>(part + D), make_float4(m, l, 0.f, 0.f));
+    __stcg(reinterpret_cast<float2*>(part - row + D / 4 * BM) + row, make_float2(m, l));
     __threadfence();
     // two flag slots alternate, so a slot is rewritten only after every thread read it
     volatile int* flag = merge_flag + (split_cnt & 1);
@@ -979,42 +986,78 @@ __device__ __forceinline__ bool softmax_group(const AttnParams& p, const Sched& 
     }
     if (*flag == 0) continue;
     __threadfence();
-    if (valid) {
-      const float* base =
-          p.ws_part + ((static_cast<int64_t>(u.item) * sc.C * 2 + X) * BM + row) * C::kPartFloats;
-      const int64_t stride = static_cast<int64_t>(2) * BM * C::kPartFloats;  // next range
-      // O = sum_c 2^(m_c - M) O_c / sum_c 2^(m_c - M) l_c, M = max_c m_c
-      float M = -INFINITY;
-      for (int c = 0; c < sc.C; ++c) M = fmaxf(M, __ldcg(base + c * stride + D));
-      float L = 0.f;
-      for (int c = 0; c < sc.C; ++c) {
-        const float2 ml = __ldcg(reinterpret_cast<const float2*>(base + c * stride + D));
-        if (!(MASKED && M == -INFINITY)) L += ml.y * ex2_approx(ml.x - M);
+    {
+      const float4* base =
+          reinterpret_cast<const float4*>(p.ws_part) +
+          (static_cast<int64_t>(u.item) * sc.C * 2 + X) * (BM * C::kPartFloats / 4) + row;
+      constexpr int64_t stride = 2 * (BM * C::kPartFloats / 4);  // next range
+      auto ml = [&](int c) {
+        return __ldcg(reinterpret_cast<const float2*>(base - row + c * stride + D / 4 * BM) + row);
+      };
+      // O = sum_c 2^(m_c - M) O_c / sum_c 2^(m_c - M) l_c, M = max_c m_c (a split launch is
+      // never block-masked: every m_c is finite)
+      // up to kMergeAhead loads per thread in flight: a merge is a chain of L2 round trips
+      constexpr int kMergeAhead = 4;
+      float M = -INFINITY, L = 0.f;
+      for (int c0 = 0; c0 < sc.C; c0 += kMergeAhead) {
+        float2 v[kMergeAhead];
+#pragma unroll
+        for (int i = 0; i < kMergeAhead; ++i) v[i] = ml(min(c0 + i, sc.C - 1));
+        float m_new = M;
+#pragma unroll
+        for (int i = 0; i < kMergeAhead; ++i) m_new = fmaxf(m_new, v[i].x);
+        L *= ex2_approx(M - m_new);
+        M = m_new;
+#pragma unroll
+        for (int i = 0; i < kMergeAhead; ++i)
+          if (c0 + i < sc.C) L += v[i].y * ex2_approx(v[i].x - M);
       }
-      const bool empty = MASKED && M == -INFINITY;  // no range saw an allowed key
-      const float inv_L = empty ? 0.f : 1.0f / L;
+      const float inv_L = 1.0f / L;
+      float acc[32];
+      auto add = [&](float wgt, const float4(&v)[8]) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          acc[4 * q] = fmaf(v[q].x, wgt, acc[4 * q]);
+          acc[4 * q + 1] = fmaf(v[q].y, wgt, acc[4 * q + 1]);
+          acc[4 * q + 2] = fmaf(v[q].z, wgt, acc[4 * q + 2]);
+          acc[4 * q + 3] = fmaf(v[q].w, wgt, acc[4 * q + 3]);
+        }
+      };
+      // two blocks of 32 columns at a time, each with two ranges, or one block with
+      // kMergeAhead ranges at a time
+      const int blocks = sc.C <= 2 ? 2 : 1, at_once = kMergeAhead / blocks;
 #pragma unroll 1
-      for (int cc = 0; cc < D / 32; ++cc) {
-        float acc[32];
+      for (int cc = 0; cc < D / 32; cc += blocks) {
 #pragma unroll
         for (int e = 0; e < 32; ++e) acc[e] = 0.f;
-        for (int c = 0; c < sc.C; ++c) {
-          const float* pc = base + c * stride;
-          const float wgt = empty ? 0.f : ex2_approx(__ldcg(pc + D) - M);
+#pragma unroll 1
+        for (int c0 = 0; c0 < sc.C; c0 += at_once) {
+          float4 v[kMergeAhead][8];
+          float m_c[kMergeAhead];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const float4 v = __ldcg(reinterpret_cast<const float4*>(pc + cc * 32) + q);
-            acc[4 * q] = fmaf(v.x, wgt, acc[4 * q]);
-            acc[4 * q + 1] = fmaf(v.y, wgt, acc[4 * q + 1]);
-            acc[4 * q + 2] = fmaf(v.z, wgt, acc[4 * q + 2]);
-            acc[4 * q + 3] = fmaf(v.w, wgt, acc[4 * q + 3]);
+          for (int i = 0; i < kMergeAhead; ++i) {
+            const int blk = blocks == 2 ? i / 2 : 0;
+            const int c = min(c0 + (blocks == 2 ? i % 2 : i), sc.C - 1);
+            m_c[i] = ml(c).x;
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+              v[i][q] = __ldcg(base + c * stride + ((cc + blk) * 8 + q) * BM);
+          }
+#pragma unroll
+          for (int i = 0; i < kMergeAhead; ++i) {
+            if (blocks == 2 && i == 2) {
+              if (valid) store_row_bf16<32>(orow + cc * 32, acc, inv_L);
+#pragma unroll
+              for (int e = 0; e < 32; ++e) acc[e] = 0.f;
+            }
+            if (c0 + (blocks == 2 ? i % 2 : i) < sc.C) add(ex2_approx(m_c[i] - M), v[i]);
           }
         }
-        store_row_bf16<32>(orow + cc * 32, acc, inv_L);
+        if (valid) store_row_bf16<32>(orow + (cc + blocks - 1) * 32, acc, inv_L);
       }
-      if (p.lse)
+      if (valid && p.lse)
         p.lse[static_cast<int64_t>(u.h) * p.S_tok + token] =
-            empty ? -INFINITY : (M + __log2f(L)) * 0.69314718055994531f;
+            (M + __log2f(L)) * 0.69314718055994531f;
     }
     if (row == 0) p.ws_count[2 * u.item + X] = 0;  // ready for the next launch
   }
