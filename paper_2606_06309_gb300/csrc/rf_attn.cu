@@ -146,6 +146,7 @@ struct AttnParams {
   float* ws_part;  // [kMaxGrid][2][BM][D+4] partial rows
   const uint8_t* block_mask;  // [H][nkv][nkv] token block mask (128-token blocks), or null
   const int* lpt_order;       // (block mask, with a workspace) unit order for the queue, or null
+  uint32_t* lpt_bits;         // (with lpt_order) the items' tile bitmaps, or null: scan the mask
   int lpt_heads_l2;           // heads whose K/V fit in half of L2 (at least 1)
   int lpt_grid;               // CTAs of the attention launch
   int64_t o_row_stride;
@@ -261,6 +262,33 @@ __device__ __forceinline__ QRanges unit_qranges(const AttnParams& p, const Sched
     r = seg_end;
   }
   return q;
+}
+
+// One warp: word k0 + lane of the bitmap of the KV tiles that some query block of the ranges may
+// attend to, each lane loading independent mask bytes.
+__device__ __forceinline__ uint32_t kept_words(const AttnParams& p, const QRanges& q, int k0) {
+  const int lane = threadIdx.x & 31;
+  const int words = min(32, ((p.nkv + 31) >> 5) - k0);
+  // bit l of acc: may some query block attend to tile (k0 + l) * 32 + lane?
+  uint32_t acc = 0;
+  for (int i = 0; i < q.n; ++i)
+    for (int qb = q.lo[i]; qb <= q.hi[i]; ++qb) {
+      const uint8_t* mrow = q.mh + static_cast<int64_t>(qb) * p.nkv;
+#pragma unroll 1
+      for (int l0 = 0; l0 < words; l0 += 8)
+#pragma unroll
+        for (int l = 0; l < 8; ++l) {
+          const int j = (k0 + l0 + l) * 32 + lane;
+          if (j < p.nkv && mrow[j] != 0) acc |= 1u << (l0 + l);
+        }
+    }
+  // transpose: lane l collects word k0 + l (tiles (k0 + l) * 32 .. + 31)
+  uint32_t mine = 0;
+  for (int l = 0; l < words; ++l) {
+    const uint32_t bits = __ballot_sync(0xffffffffu, (acc >> l) & 1u);
+    if (lane == l) mine = bits;
+  }
+  return mine;
 }
 
 // First set bit at or after j in a unit's tile bitmap of nw words; nw * 32 (>= nkv) if none.
@@ -413,29 +441,21 @@ __device__ __forceinline__ void tile_list_builder(const AttnParams& p, const Sch
       return;
     }
     const Unit u = get_unit(sc, p, w);
-    const QRanges q = unit_qranges(p, sc, u);
     int total = 0;
-    for (int k0 = 0; k0 < nw; k0 += 32) {
-      // bit l of acc: may some query block of the unit attend to tile (k0 + l) * 32 + lane?
-      uint32_t acc = 0;
-      for (int i = 0; i < q.n; ++i)
-        for (int qb = q.lo[i]; qb <= q.hi[i]; ++qb) {
-          const uint8_t* mrow = q.mh + static_cast<int64_t>(qb) * p.nkv;
-#pragma unroll
-          for (int l = 0; l < 32; ++l) {
-            const int j = (k0 + l) * 32 + lane;
-            if (j < p.nkv && mrow[j] != 0) acc |= 1u << l;
-          }
-        }
-      // transpose: lane l collects word k0 + l (tiles (k0 + l) * 32 .. + 31)
-      uint32_t mine = 0;
-#pragma unroll
-      for (int l = 0; l < 32; ++l) {
-        const uint32_t bits = __ballot_sync(0xffffffffu, (acc >> l) & 1u);
-        if (lane == l) mine = bits;
+    if (p.lpt_bits != nullptr) {
+      // the pre-pass has built the bitmaps of all items
+      for (int i = lane; i < nw; i += 32) {
+        const uint32_t x = p.lpt_bits[static_cast<int64_t>(w) * nw + i];
+        words[i] = x;
+        total += __popc(x);
       }
-      if (k0 + lane < nw) words[k0 + lane] = mine;
-      total += __popc(mine);  // zero for words past nw: their tiles are >= nkv
+    } else {
+      const QRanges q = unit_qranges(p, sc, u);
+      for (int k0 = 0; k0 < nw; k0 += 32) {
+        const uint32_t mine = kept_words(p, q, k0);
+        if (k0 + lane < nw) words[k0 + lane] = mine;
+        total += __popc(mine);  // zero for words past nw: their tiles are >= nkv
+      }
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) total += __shfl_xor_sync(0xffffffffu, total, off);
@@ -1203,8 +1223,10 @@ __device__ __forceinline__ int lpt_group_heads(const AttnParams& p, const Sched&
 }
 //
 // Each CTA covers kPrepassItems items of one head, one warp per item: the item's cost is the
-// number of set bits of the bitmap the builder will write, found with each lane loading 32
-// independent mask bytes per query block.  The CTA that completes a group (a counter per group
+// number of set bits of its bitmap of KV tiles (kept_words), which is kept in the workspace for
+// the CTA that takes the item.  (With the mask scanned again by every CTA for every item it
+// takes, and 4097 bins in the sort whatever the number of key blocks, the keyframe-only step of
+// 13 x 1560 tokens under a banded mask took 145 us instead of 140.5.)  The CTA that completes a group (a counter per group
 // in the workspace, reset by that CTA) sorts the group by decreasing cost with a counting sort.
 // The order among equal costs is arbitrary, which changes no result (every item is computed
 // the same way by whichever CTA takes it) and, within an L2-sized group, no locality.
@@ -1212,12 +1234,11 @@ constexpr int kPrepassItems = 8;       // items (warps) per CTA
 constexpr int kPrepassThreads = 32 * kPrepassItems;
 constexpr int kQueueGroup0 = 2;        // first per-group counter word
 constexpr int kMaxLptGroups = kMaxGrid - kQueueGroup0;
-constexpr int kCostBins = kTLMaxTiles + 1;
-constexpr int kBinsPerThread = (kCostBins + kPrepassThreads - 1) / kPrepassThreads;
+constexpr int kMaxBins = (kTLMaxTiles / kPrepassThreads + 1) * kPrepassThreads;
 
 __global__ void __launch_bounds__(kPrepassThreads)
     lpt_prepass_kernel(const AttnParams p, int* cost, int* order, int ctas_per_head) {
-  __shared__ int start[kBinsPerThread * kPrepassThreads];  // bin b holds cost kTLMaxTiles - b
+  __shared__ int start[kMaxBins];
   __shared__ int warp_sum[kPrepassThreads / 32];
   __shared__ int last;
   const Sched sc = make_sched(p);  // a block-masked launch: no split, so units are items
@@ -1237,17 +1258,10 @@ __global__ void __launch_bounds__(kPrepassThreads)
     const int nw = (p.nkv + 31) >> 5;
     int total = 0;
     for (int k0 = 0; k0 < nw; k0 += 32) {
-      uint32_t acc = 0;  // bit l: tile (k0 + l) * 32 + lane allowed
-      for (int i = 0; i < q.n; ++i)
-        for (int qb = q.lo[i]; qb <= q.hi[i]; ++qb) {
-          const uint8_t* mrow = q.mh + static_cast<int64_t>(qb) * p.nkv;
-#pragma unroll
-          for (int l = 0; l < 32; ++l) {
-            const int j = (k0 + l) * 32 + lane;
-            if (j < p.nkv && mrow[j] != 0) acc |= 1u << l;
-          }
-        }
-      total += __popc(acc);
+      const uint32_t mine = kept_words(p, q, k0);
+      if (p.lpt_bits != nullptr && k0 + lane < nw)
+        p.lpt_bits[static_cast<int64_t>(base + item) * nw + k0 + lane] = mine;
+      total += __popc(mine);
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) total += __shfl_xor_sync(0xffffffffu, total, off);
@@ -1267,20 +1281,18 @@ __global__ void __launch_bounds__(kPrepassThreads)
   __syncthreads();
   if (!last) return;
   __threadfence();
-  for (int i = tid; i < kBinsPerThread * kPrepassThreads; i += kPrepassThreads) start[i] = 0;
+  // bin b holds the items with nkv - b tiles: only as many bins as an item can have tiles
+  const int bins_per_thread = p.nkv / kPrepassThreads + 1;
+  const int first_bin = tid * bins_per_thread;
+  for (int i = tid; i < bins_per_thread * kPrepassThreads; i += kPrepassThreads) start[i] = 0;
   __syncthreads();
   for (int i = tid; i < n; i += kPrepassThreads)
-    atomicAdd(&start[kTLMaxTiles - __ldcg(cost + base + i)], 1);
+    atomicAdd(&start[p.nkv - __ldcg(cost + base + i)], 1);
   __syncthreads();
-  // exclusive prefix sum over the bins: kBinsPerThread consecutive bins per thread, then a
+  // exclusive prefix sum over the bins: bins_per_thread consecutive bins per thread, then a
   // block-wide scan of the per-thread sums
-  int own[kBinsPerThread];
   int sum = 0;
-#pragma unroll
-  for (int b = 0; b < kBinsPerThread; ++b) {
-    own[b] = start[tid * kBinsPerThread + b];
-    sum += own[b];
-  }
+  for (int b = 0; b < bins_per_thread; ++b) sum += start[first_bin + b];
   int incl = sum;
 #pragma unroll
   for (int off = 1; off < 32; off <<= 1) {
@@ -1300,14 +1312,14 @@ __global__ void __launch_bounds__(kPrepassThreads)
   }
   __syncthreads();
   int run = incl - sum + (wid > 0 ? warp_sum[wid - 1] : 0);
-#pragma unroll
-  for (int b = 0; b < kBinsPerThread; ++b) {
-    start[tid * kBinsPerThread + b] = run;
-    run += own[b];
+  for (int b = 0; b < bins_per_thread; ++b) {
+    const int own = start[first_bin + b];
+    start[first_bin + b] = run;
+    run += own;
   }
   __syncthreads();
   for (int i = tid; i < n; i += kPrepassThreads)
-    order[base + atomicAdd(&start[kTLMaxTiles - __ldcg(cost + base + i)], 1)] = base + i;
+    order[base + atomicAdd(&start[p.nkv - __ldcg(cost + base + i)], 1)] = base + i;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1472,6 +1484,7 @@ rf_status attn_impl(void* d_O, float* d_lse, const void* d_Q, const void* d_K, c
                     : nullptr;
   p.block_mask = d_block_mask;
   p.lpt_order = nullptr;
+  p.lpt_bits = nullptr;
   p.lpt_heads_l2 = 1;
   p.lpt_grid = 0;
   p.o_row_stride = o_row_stride;
@@ -1494,6 +1507,10 @@ rf_status attn_impl(void* d_O, float* d_lse, const void* d_Q, const void* d_K, c
         2 * max_items * 4 <= workspace_bytes(d, grid) - kCountBytes) {
       int* cost = reinterpret_cast<int*>(p.ws_part);
       int* order = cost + max_items;
+      // the items' tile bitmaps after them, where there is room (else the CTAs scan the mask again)
+      const int64_t words = (p.nkv + 31) / 32;
+      if ((2 + words) * max_items * 4 <= workspace_bytes(d, grid) - kCountBytes)
+        p.lpt_bits = reinterpret_cast<uint32_t*>(order + max_items);
       p.lpt_heads_l2 = static_cast<int>(std::min<int64_t>(heads_l2, H));
       p.lpt_grid = grid;
       const int per_head = static_cast<int>((max_pairs + kPrepassItems - 1) / kPrepassItems);
