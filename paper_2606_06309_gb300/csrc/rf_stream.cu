@@ -200,7 +200,16 @@ __global__ void __launch_bounds__(kStreamThreads)
 // active[a], whose fresh rows are stored into its cache's other slot (shift-and-store); the
 // rest are skipped[a - A], whose rows are rewritten with Eq. 3 from the two cached states.
 // Eight bf16 per 16-byte access; fp32 arithmetic, rounded to nearest even.
+//
+// Bound by HBM.  Every frame has work, so the grid has one CTA per chunk of 128 threads x 4 vectors
+// (8 KB of each stream) and the scheduler deals them out; walking the chunks with a fixed grid of
+// four CTAs of 256 threads per SM left the SMs' last chunks uneven.  Keyframe-only step of
+// 33 x 3600 x 3072: 595 -> 570 us (7.2 TB/s; 7.1 TB/s is what torch.add's two reads and a
+// write reach), all frames active 435 -> 405 us, 13 x 1560 x 1536: 52.1 -> 50.0 us.  256 threads
+// 567 / 422 / 50.9, two or eight vectors per thread at 256 threads 568 / 414 / 50.2 and
+// 676 / 522 / 59.8.
 // ---------------------------------------------------------------------------------------
+constexpr int kKvThreads = 128;
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
 __device__ __forceinline__ uint32_t proj_pair(uint32_t cur, uint32_t prev, float a, float b) {
@@ -211,7 +220,7 @@ __device__ __forceinline__ uint32_t proj_pair(uint32_t cur, uint32_t prev, float
   return r;
 }
 
-__global__ void __launch_bounds__(kStreamThreads)
+__global__ void __launch_bounds__(kKvThreads)
     project_kv_kernel(uint16_t* __restrict__ K, uint16_t* __restrict__ V, int64_t row_stride,
                       uint16_t* __restrict__ Kc, uint16_t* __restrict__ Vc,
                       const uint8_t* __restrict__ cur_slot, const float* __restrict__ alpha,
@@ -224,7 +233,7 @@ __global__ void __launch_bounds__(kStreamThreads)
   A = A < 0 ? 0 : (A > F ? F : A);
   const int D8 = D >> 3;                      // 16-byte vectors per row
   const int64_t frame_vecs = static_cast<int64_t>(N) * D8;
-  constexpr int64_t kChunk = static_cast<int64_t>(kStreamThreads) * kUnroll;
+  constexpr int64_t kChunk = static_cast<int64_t>(kKvThreads) * kUnroll;
   const int64_t per_frame = (frame_vecs + kChunk - 1) / kChunk;
   const int64_t total = per_frame * F;
   const int64_t slot_stride = static_cast<int64_t>(F) * N * D;  // elements between slots
@@ -252,9 +261,9 @@ __global__ void __launch_bounds__(kStreamThreads)
       }
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
-        off[u] = contiguous ? base + u * kStreamThreads : p * (row_stride >> 3) + q;
+        off[u] = contiguous ? base + u * kKvThreads : p * (row_stride >> 3) + q;
         if (!contiguous) {
-          q += kStreamThreads;
+          q += kKvThreads;
           while (q >= D8) {
             q -= D8;
             ++p;
@@ -267,10 +276,10 @@ __global__ void __launch_bounds__(kStreamThreads)
       uint4 x[kUnroll];
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u)
-        if (base + u * kStreamThreads < frame_vecs) x[u] = __ldcs(rv + off[u]);
+        if (base + u * kKvThreads < frame_vecs) x[u] = __ldcs(rv + off[u]);
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
-        const int64_t v = base + u * kStreamThreads;
+        const int64_t v = base + u * kKvThreads;
         if (v < frame_vecs) __stcs(prev + v, x[u]);  // the other slot
       }
     } else {
@@ -278,7 +287,7 @@ __global__ void __launch_bounds__(kStreamThreads)
       uint4 x[kUnroll], y[kUnroll];
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
-        const int64_t v = base + u * kStreamThreads;
+        const int64_t v = base + u * kKvThreads;
         if (v < frame_vecs) {
           x[u] = __ldcs(cur + v);
           y[u] = __ldcs(prev + v);
@@ -286,7 +295,7 @@ __global__ void __launch_bounds__(kStreamThreads)
       }
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
-        if (base + u * kStreamThreads < frame_vecs) {
+        if (base + u * kKvThreads < frame_vecs) {
           uint4 r;
           r.x = proj_pair(x[u].x, y[u].x, al, be);
           r.y = proj_pair(x[u].y, y[u].y, al, be);
@@ -393,11 +402,11 @@ extern "C" rf_status rf_project_kv(void* d_K, void* d_V, int64_t kv_row_stride, 
   DeviceInfo di;
   if (rf_status st = current_device_info(&di)) return st;
   const int64_t frame_vecs = static_cast<int64_t>(N) * (D / 8);
-  const int64_t chunk = static_cast<int64_t>(kStreamThreads) * kUnroll;
+  const int64_t chunk = static_cast<int64_t>(kKvThreads) * kUnroll;
   int64_t blocks = ((frame_vecs + chunk - 1) / chunk) * F;
-  if (blocks > 4LL * di.sm_count) blocks = 4LL * di.sm_count;
+  if (blocks > 0x7FFFFFFFLL) blocks = 0x7FFFFFFFLL;  // the kernel walks on from there
   dim3 grid(static_cast<unsigned>(blocks), 2);
-  project_kv_kernel<<<grid, kStreamThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+  project_kv_kernel<<<grid, kKvThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
       static_cast<uint16_t*>(d_K), static_cast<uint16_t*>(d_V), kv_row_stride,
       static_cast<uint16_t*>(d_Kc), static_cast<uint16_t*>(d_Vc), d_cur_slot, d_alpha, d_beta,
       d_active, d_skipped, d_counts, F, N, D);
