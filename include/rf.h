@@ -186,11 +186,14 @@ rf_status rf_project_kv(void* d_K, void* d_V, int64_t kv_row_stride, void* d_Kc,
  *   d_workspace, workspace_bytes  optional device scratch for split-KV (NULL / 0 =
  *                no split).  With at least rf_attn_workspace_bytes(d) bytes, 256-byte
  *                aligned and ZERO-FILLED before its first use, the last, partly
- *                idle round of work is split into ranges of keys whose partial
- *                results are merged on the device; the kernel leaves the workspace
- *                ready for the next call.  Calls that share a workspace must not
- *                overlap on the GPU (keep them on one stream).  After a call that
- *                reported RF_ERR_DEVICE_TIMEOUT, zero it again.
+ *                idle round of work is shared out over ranges of keys whose partial
+ *                results are merged on the device, in a fixed order; the kernel leaves
+ *                the workspace ready for the next call.  A buffer of 4096 bytes plus half
+ *                of the rest is taken too, but only splits a round in which at least
+ *                half of the SMs would idle; a smaller one is not used.
+ *                Calls that share a workspace must not overlap on the GPU (keep them
+ *                on one stream).  After a call that reported RF_ERR_DEVICE_TIMEOUT,
+ *                zero it again.
  * Requires an sm_103 device; bases 16-byte aligned.
  */
 rf_status rf_attn(void* d_O, float* d_lse, const void* d_Q, const void* d_K, const void* d_V,
@@ -214,9 +217,9 @@ rf_status rf_attn(void* d_O, float* d_lse, const void* d_Q, const void* d_K, con
  * with a workspace (same size and rules as for rf_attn) a small pre-pass launch orders the
  * work items longest first within groups of heads and the CTAs take them from a queue.  The
  * queue and the groups use the workspace's counter words, which the calls leave at zero, and
- * the items' costs and order use its partial-row area.  Without a workspace, items are dealt
- * round-robin.  Returns RF_ERR_INVALID_ARG for a null mask and RF_ERR_UNSUPPORTED for more
- * than 4096 key blocks (F*N > 524288 tokens).
+ * the items' costs, order and key-block bitmaps use its partial-row area.  Without a
+ * workspace, items are dealt round-robin.  Returns RF_ERR_INVALID_ARG for a null mask and
+ * RF_ERR_UNSUPPORTED for more than 4096 key blocks (F*N > 524288 tokens).
  */
 rf_status rf_attn_block_masked(void* d_O, float* d_lse, const void* d_Q, const void* d_K,
                                const void* d_V, int64_t qkv_row_stride, int64_t o_row_stride,
@@ -227,9 +230,9 @@ rf_status rf_attn_block_masked(void* d_O, float* d_lse, const void* d_Q, const v
 
 /*
  * rf_attn_workspace_bytes -- bytes of split-KV workspace rf_attn can use on the
- * current device for head dim d (independent of the problem size: counters plus
- * one partial result tile per SM).  Returns -1 for an unsupported d or when the
- * device cannot be queried.
+ * current device for head dim d (independent of the problem size: 4096 bytes of
+ * counters plus the partial results of two pieces of work per SM).  Returns -1 for an
+ * unsupported d or when the device cannot be queried.
  */
 int64_t rf_attn_workspace_bytes(int d);
 
@@ -243,7 +246,7 @@ int64_t rf_attn_workspace_bytes(int d);
  * C hosts with no device allocator of their own.  For them this call takes the
  * same arguments as rf_attn minus the workspace, and uses instead a scratch
  * array that the library itself holds in device memory: a file-scope array of
- * 21,630,976 bytes (split-KV counters plus partial tiles for head dim <= 128 on
+ * 43,257,856 bytes (split-KV counters plus partial tiles for head dim <= 128 on
  * up to 160 SMs), present on every GPU that loads the library until the
  * process exits.  The call allocates and frees nothing.
  *   - The first call on a device looks up the array's device address

@@ -44,11 +44,11 @@
 // (each frame padded to a multiple of 8 rows); items are dealt round-robin to the CTAs, so
 // consecutive CTAs share the same head's K/V through L2 (block-masked launches with a
 // workspace take items from a longest-first work queue instead).  When the last round of items
-// would leave more than half of the CTAs idle and the caller supplied a workspace, each item of
-// that round is split into C ranges of KV tiles (split-KV, unmasked launches only): every range
-// writes its unnormalised O row, running max and sum to the workspace, and the CTA that
-// finishes the last range of an item merges them (counter per item and query tile, reset to
-// zero by the merging CTA).
+// leaves CTAs idle and the caller supplied a workspace, it is shared out by KV tiles (split-KV,
+// unmasked launches only; make_sched has the rule): each item in C equal ranges, or all CTAs equal
+// shares of the round.  Every range of a split item writes its unnormalised O rows, running max
+// and sum to the workspace, and the CTA that finishes the last range of an item merges them in
+// the order of the ranges (counter per item and query tile, reset to zero by the merging CTA).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -143,7 +143,8 @@ struct AttnParams {
   const int32_t* counts;
   int32_t* status;
   int* ws_count;   // [kMaxGrid] merge counters (zero between launches), or null: no split
-  float* ws_part;  // [kMaxGrid][2][BM][D+4] partial rows
+  float* ws_part;  // [ws_slots * CTAs][2] tiles of partial rows
+  int ws_slots;    // partial slots per CTA
   const uint8_t* block_mask;  // [H][nkv][nkv] token block mask (128-token blocks), or null
   const int* lpt_order;       // (block mask, with a workspace) unit order for the queue, or null
   uint32_t* lpt_bits;         // (with lpt_order) the items' tile bitmaps, or null: scan the mask
@@ -159,15 +160,41 @@ struct Sched {
   int R, tiles, pairs;  // active rows (padded per frame), query tiles and tile pairs per head
   int T_full;           // items processed whole
   int C;                // KV ranges per item of the split tail (1: no split)
-  int units;            // T_full + tail items * C
+  uint32_t even_q, even_r;  // the tail dealt out evenly: its KV tiles / CTAs and the remainder (0: not)
+  int units;            // T_full + tail items * C, or + 2 per CTA (some empty) when dealt evenly
 };
 
 // One unit of work: a tile pair of one head over KV tiles [j0, j1).
 struct Unit {
   int h, pr, j0, j1;
-  int part;  // split: partial slot (tail item index * C + range), else -1
+  int part;  // split: partial slot, else -1
   int item;  // split: tail item index
 };
+
+// How the last, partly idle round of items is shared out (unmasked launches with a workspace),
+// chosen by the KV tiles that the busiest CTA then processes:
+//   whole        nkv
+//   C ranges     nkv / C + kSplitCost, C = CTAs / items: every item in equal ranges, one per CTA
+//   dealt evenly tail * nkv / CTAs + kEvenCost: every CTA takes the same share of the tail's KV tiles,
+//                which may end in one item and begin the next (needs two partial slots per CTA)
+// The costs are the boundary of a further unit and the merge, in KV tiles (dealt evenly, the
+// partials of all items are written and read: 34 MB each way for 100 items on 152 CTAs, some 10 us).
+// Dealing evenly is considered where C ranges leave CTAs idle: more than a quarter as many items as
+// CTAs (below, the items' ranges fill the chip and an item would be in more than five pieces).
+// Measured (us per launch, whole or in C ranges -> dealt evenly): 13 x 1560 tokens x 1 head x 128
+// (80 items) 186 -> 122; 9 of the 13 frames active (55 items) 107 -> 93; 7 x 1003 x 5 x 128, 5 active
+// (100 items of 55 tiles) 70.3 -> 66.9.
+constexpr int kSplitCost = 3, kEvenCost = 10;
+constexpr uint32_t kMinEvenShare = 12;  // KV tiles per CTA
+// KV tile, counted over the whole tail, where CTA k's share begins; no piece is shorter than
+// kMinSplitTiles.
+__device__ __forceinline__ uint32_t even_bound(const Sched& s, int nkv, int k) {
+  // (fits 32 bits: the tail has fewer items than CTAs, and make_sched checks CTAs * nkv)
+  const uint32_t v = k * s.even_q + k * s.even_r / gridDim.x;
+  const uint32_t rem = v % static_cast<uint32_t>(nkv);
+  if (rem < kMinSplitTiles) return v - rem;
+  return nkv - rem < kMinSplitTiles ? v + (nkv - rem) : v;
+}
 
 __device__ __forceinline__ Sched make_sched(const AttnParams& p) {
   int A = p.counts[0];
@@ -180,6 +207,7 @@ __device__ __forceinline__ Sched make_sched(const AttnParams& p) {
   const int G = gridDim.x;
   s.T_full = T;
   s.C = 1;
+  s.even_q = s.even_r = 0;
   // Block-masked launches never split: their items differ in cost, so the makespan of the
   // static assignment is set by the costliest CTA rather than by the last round's tail, and a
   // split only adds the merge (measured slower on the 13 x 1560-token workload).
@@ -189,6 +217,17 @@ __device__ __forceinline__ Sched make_sched(const AttnParams& p) {
     int c = G / tail;
     if (c > kMaxSplit) c = kMaxSplit;
     if (c > p.nkv / kMinSplitTiles) c = p.nkv / kMinSplitTiles;
+    const int busiest = c >= 2 ? (p.nkv + c - 1) / c + kSplitCost : p.nkv;
+    if (p.ws_slots == 2 && 4 * tail > G && static_cast<uint32_t>(p.nkv) <= 0xFFFFFFFFu / G) {
+      const uint32_t all = static_cast<uint32_t>(tail) * p.nkv, q = all / G;
+      if (q >= kMinEvenShare && static_cast<int>(q) + 1 + kEvenCost < busiest) {
+        s.T_full = (rounds - 1) * G;
+        s.even_q = q;
+        s.even_r = all % G;
+        s.units = s.T_full + 2 * G;
+        return s;
+      }
+    }
     if (c >= 2) {
       s.T_full = (rounds - 1) * G;
       s.C = c;
@@ -201,12 +240,33 @@ __device__ __forceinline__ Sched make_sched(const AttnParams& p) {
 __device__ __forceinline__ Unit get_unit(const Sched& s, const AttnParams& p, int w) {
   Unit u;
   int item;
+  u.part = -1;
+  u.item = -1;
   if (w < s.T_full) {
     item = w;
     u.j0 = 0;
     u.j1 = p.nkv;
-    u.part = -1;
-    u.item = -1;
+  } else if (s.even_q != 0) {
+    // the CTA's share of the tail: what is left of the item it begins in, then the start of the
+    // next one (perhaps nothing: j1 = 0).  A share is shorter than an item.
+    const int G = gridDim.x;
+    int k = w - s.T_full;
+    const bool second = k >= G;
+    if (second) k -= G;
+    const uint32_t lo = even_bound(s, p.nkv, k), hi = even_bound(s, p.nkv, k + 1);
+    const uint32_t first = lo / static_cast<uint32_t>(p.nkv);
+    const uint32_t begin = first * p.nkv, end = begin + p.nkv;
+    if (!second) {
+      u.item = static_cast<int>(first);
+      u.j0 = static_cast<int>(lo - begin);
+      u.j1 = static_cast<int>(min(hi, end) - begin);
+    } else {
+      u.item = static_cast<int>(first) + 1;
+      u.j0 = 0;
+      u.j1 = hi > end ? static_cast<int>(hi - end) : 0;
+    }
+    item = s.T_full + u.item;
+    if (u.j1 - u.j0 < p.nkv) u.part = 2 * k + second;
   } else {
     const int k = w - s.T_full;
     const int ti = k / s.C, c = k - ti * s.C;
@@ -220,7 +280,30 @@ __device__ __forceinline__ Unit get_unit(const Sched& s, const AttnParams& p, in
   }
   u.h = item / s.pairs;
   u.pr = item - u.h * s.pairs;
+  if (u.j0 >= u.j1) u.pr = s.pairs;  // an empty share: neither query tile exists
   return u;
+}
+
+// The partial slots of a split item, in the order of their KV ranges: slot `first`, then
+// `rest + c * stride` for c = 1 .. n - 1.
+struct Pieces {
+  int n, first, rest, stride;
+};
+__device__ __forceinline__ Pieces item_pieces(const Sched& s, const AttnParams& p, const Unit& u) {
+  if (s.even_q == 0) return Pieces{s.C, u.item * s.C, u.item * s.C, 1};
+  // the CTAs whose shares meet the item: from the last that begins at or before it ...
+  const uint32_t begin = static_cast<uint32_t>(u.item) * p.nkv, end = begin + p.nkv;
+  const int G = gridDim.x;
+  int k0 = min(G - 1, static_cast<int>(static_cast<float>(begin) /
+                                       (static_cast<float>(s.even_q) +
+                                        static_cast<float>(s.even_r) / static_cast<float>(G))));
+  while (k0 > 0 && even_bound(s, p.nkv, k0) > begin) --k0;
+  while (even_bound(s, p.nkv, k0 + 1) <= begin) ++k0;
+  // ... to the first that ends at or after its end
+  int k1 = k0;
+  while (even_bound(s, p.nkv, k1 + 1) < end) ++k1;
+  const bool second = even_bound(s, p.nkv, k0) < begin;  // its share began in the item before
+  return Pieces{k1 - k0 + 1, 2 * k0 + second, 2 * k0, 2};
 }
 
 // Token block mask (combined frame x token mask).  The valid query rows of a unit's tile pair
@@ -680,8 +763,8 @@ __device__ __forceinline__ bool mma_issuer(const AttnParams& p, const Sched& sc,
     // number of KV tiles of the unit: j1 - j0, or (MASKED) the set bits of the builder's
     // bitmap (the issuer needs only the count; the producer walks the bits)
     const int ntiles = MASKED ? static_cast<int>(tw[kTLWords]) : u.j1 - u.j0;
-    if (X == 1 && !hasB) {
-      // no second query tile: only give the K/V slots back
+    if (2 * u.pr + X >= sc.tiles) {
+      // no such query tile: only give the K/V slots back
       bool ok = true;
       for (int i = 0; ok && i < 2 * ntiles; ++i, ++it) {
         ok = wait_slot(it);
@@ -779,6 +862,124 @@ __device__ __forceinline__ void store_row_bf16(uint16_t* orow, const float* o, f
     v.w = pack_bf16x2(o[8 * q + 6] * scale, o[8 * q + 7] * scale);
     dst[q] = v;
   }
+}
+
+// The end of a split item's KV range, for the 128 threads of a softmax warpgroup (thread = row):
+// publish the partial rows; the last range to finish merges them all.  Returns 0, or where a wait
+// gave up.  Out of line: it is rare, and inlined it changes how the softmax loop is compiled.
+template <int D>
+__device__ __noinline__ int split_epilogue(const AttnParams& p, const Sched& sc, const Unit& u, int X,
+                                           int row, uint32_t tO, float m, float l, int64_t token,
+                                           uint32_t bar, int g_cnt, volatile int* abort,
+                                           volatile int* flag) {
+  using C = Cfg<D>;
+  const bool valid = token >= 0;
+  uint16_t* orow = p.O + token * p.o_row_stride + static_cast<int64_t>(u.h) * D;
+  // A tile's partials are [D/4] float4 columns of 128 rows, then {m, l} of the rows: a warp's
+  // stores and loads are 512 consecutive bytes.  (With each row's 528 bytes together and one
+  // range at a time in the merge, 4 x 256 tokens x 2 heads x 128 in 8 ranges took 69 us, now in 2
+  // ranges 17.6; 7 x 1003 x 2 x 128 in 7 ranges 69.6 -> 45.9.)
+  float4* part = reinterpret_cast<float4*>(p.ws_part) +
+                 static_cast<int64_t>(u.part * 2 + X) * (BM * C::kPartFloats / 4) + row;
+#pragma unroll 1
+  for (int c = 0; c < D / 32; ++c) {
+    uint32_t o[32];
+    tmem_ld32(tO + c * 32, o);
+    tmem_wait_ld();
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      __stcg(part + (c * 8 + q) * BM,
+             make_float4(__uint_as_float(o[4 * q]), __uint_as_float(o[4 * q + 1]),
+                         __uint_as_float(o[4 * q + 2]), __uint_as_float(o[4 * q + 3])));
+  }
+  __stcg(reinterpret_cast<float2*>(part - row + D / 4 * BM) + row, make_float2(m, l));
+  __threadfence();
+  if (!group_sync(bar, g_cnt, abort)) return 5;  // every row is published
+  const Pieces pieces = item_pieces(sc, p, u);
+  if (row == 0) {
+    const int old = atomicAdd(p.ws_count + 2 * u.item + X, 1);
+    *flag = (old == pieces.n - 1);
+  }
+  if (!group_sync(bar, g_cnt, abort)) return 6;  // the flag is visible
+  if (*flag == 0) return 0;
+  __threadfence();
+  {
+    constexpr int64_t kSlot = 2 * (BM * C::kPartFloats / 4);  // float4s
+    const float4* base =
+        reinterpret_cast<const float4*>(p.ws_part) + X * (BM * C::kPartFloats / 4) + row;
+    auto range = [&](int c) {
+      return base + (c == 0 ? pieces.first : pieces.rest + c * pieces.stride) * kSlot;
+    };
+    auto ml = [&](int c) {
+      return __ldcg(reinterpret_cast<const float2*>(range(c) - row + D / 4 * BM) + row);
+    };
+    // O = sum_c 2^(m_c - M) O_c / sum_c 2^(m_c - M) l_c, M = max_c m_c (a split launch is
+    // never block-masked: every m_c is finite)
+    // up to kMergeAhead loads per thread in flight: a merge is a chain of L2 round trips
+    constexpr int kMergeAhead = 4;
+    float M = -INFINITY, L = 0.f;
+    for (int c0 = 0; c0 < pieces.n; c0 += kMergeAhead) {
+      float2 v[kMergeAhead];
+#pragma unroll
+      for (int i = 0; i < kMergeAhead; ++i) v[i] = ml(min(c0 + i, pieces.n - 1));
+      float m_new = M;
+#pragma unroll
+      for (int i = 0; i < kMergeAhead; ++i) m_new = fmaxf(m_new, v[i].x);
+      L *= ex2_approx(M - m_new);
+      M = m_new;
+#pragma unroll
+      for (int i = 0; i < kMergeAhead; ++i)
+        if (c0 + i < pieces.n) L += v[i].y * ex2_approx(v[i].x - M);
+    }
+    const float inv_L = 1.0f / L;
+    float acc[32];
+    auto add = [&](float wgt, const float4(&v)[8]) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        acc[4 * q] = fmaf(v[q].x, wgt, acc[4 * q]);
+        acc[4 * q + 1] = fmaf(v[q].y, wgt, acc[4 * q + 1]);
+        acc[4 * q + 2] = fmaf(v[q].z, wgt, acc[4 * q + 2]);
+        acc[4 * q + 3] = fmaf(v[q].w, wgt, acc[4 * q + 3]);
+      }
+    };
+    // two blocks of 32 columns at a time, each with two ranges, or one block with
+    // kMergeAhead ranges at a time
+    const int blocks = pieces.n <= 2 ? 2 : 1, at_once = kMergeAhead / blocks;
+#pragma unroll 1
+    for (int cc = 0; cc < D / 32; cc += blocks) {
+#pragma unroll
+      for (int e = 0; e < 32; ++e) acc[e] = 0.f;
+#pragma unroll 1
+      for (int c0 = 0; c0 < pieces.n; c0 += at_once) {
+        float4 v[kMergeAhead][8];
+        float m_c[kMergeAhead];
+#pragma unroll
+        for (int i = 0; i < kMergeAhead; ++i) {
+          const int blk = blocks == 2 ? i / 2 : 0;
+          const int c = min(c0 + (blocks == 2 ? i % 2 : i), pieces.n - 1);
+          m_c[i] = ml(c).x;
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            v[i][q] = __ldcg(range(c) + ((cc + blk) * 8 + q) * BM);
+        }
+#pragma unroll
+        for (int i = 0; i < kMergeAhead; ++i) {
+          if (blocks == 2 && i == 2) {
+            if (valid) store_row_bf16<32>(orow + cc * 32, acc, inv_L);
+#pragma unroll
+            for (int e = 0; e < 32; ++e) acc[e] = 0.f;
+          }
+          if (c0 + (blocks == 2 ? i % 2 : i) < pieces.n) add(ex2_approx(m_c[i] - M), v[i]);
+        }
+      }
+      if (valid) store_row_bf16<32>(orow + (cc + blocks - 1) * 32, acc, inv_L);
+    }
+    if (valid && p.lse)
+      p.lse[static_cast<int64_t>(u.h) * p.S_tok + token] =
+          (M + __log2f(L)) * 0.69314718055994531f;
+  }
+  if (row == 0) p.ws_count[2 * u.item + X] = 0;  // ready for the next launch
+  return 0;
 }
 
 template <int D, bool MASKED>
@@ -979,117 +1180,16 @@ __device__ __forceinline__ bool softmax_group(const AttnParams& p, const Sched& 
             (MASKED && l == 0.f) ? -INFINITY : (m + __log2f(l)) * 0.69314718055994531f;
       continue;
     }
-    // split item: publish this KV range's partial rows, then the last range to finish merges.  A
-    // tile's partials are [D/4] float4 columns of 128 rows, then {m, l} of the rows: a warp's
-    // stores and loads are 512 consecutive bytes.  (With each row's 528 bytes together and one
-    // range at a time in the merge, 4 x 256 tokens x 2 heads x 128 in 8 ranges took 69 us, now in 2
-    // ranges 17.6; 7 x 1003 x 2 x 128 in 7 ranges 69.6 -> 45.9.)
-    float4* part = reinterpret_cast<float4*>(p.ws_part) +
-                   static_cast<int64_t>(u.part * 2 + X) * (BM * C::kPartFloats / 4) + row;
-#pragma unroll 1
-    for (int c = 0; c < D / 32; ++c) {
-      uint32_t o[32];
-      tmem_ld32(tO + c * 32, o);
-      tmem_wait_ld();
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        __stcg(part + (c * 8 + q) * BM,
-               make_float4(__uint_as_float(o[4 * q]), __uint_as_float(o[4 * q + 1]),
-                           __uint_as_float(o[4 * q + 2]), __uint_as_float(o[4 * q + 3])));
-    }
-    __stcg(reinterpret_cast<float2*>(part - row + D / 4 * BM) + row, make_float2(m, l));
-    __threadfence();
+    // split item: publish this KV range's partial rows, then the last range to finish merges
     // two flag slots alternate, so a slot is rewritten only after every thread read it
-    volatile int* flag = merge_flag + (split_cnt & 1);
+    if (const int bad = split_epilogue<D>(p, sc, u, X, row, tO, m, l, valid ? token : -1,
+                                          bar(C::kBarGroup + X), g_cnt,
+                                          abort, merge_flag + (split_cnt & 1))) {
+      flag_error(p, bad);
+      return false;
+    }
+    g_cnt += 2;
     ++split_cnt;
-    if (!group_sync(bar(C::kBarGroup + X), g_cnt, abort)) {  // every row is published
-      flag_error(p, 5);
-      return false;
-    }
-    if (row == 0) {
-      const int old = atomicAdd(p.ws_count + 2 * u.item + X, 1);
-      *flag = (old == sc.C - 1);
-    }
-    if (!group_sync(bar(C::kBarGroup + X), g_cnt, abort)) {  // the flag is visible
-      flag_error(p, 6);
-      return false;
-    }
-    if (*flag == 0) continue;
-    __threadfence();
-    {
-      const float4* base =
-          reinterpret_cast<const float4*>(p.ws_part) +
-          (static_cast<int64_t>(u.item) * sc.C * 2 + X) * (BM * C::kPartFloats / 4) + row;
-      constexpr int64_t stride = 2 * (BM * C::kPartFloats / 4);  // next range
-      auto ml = [&](int c) {
-        return __ldcg(reinterpret_cast<const float2*>(base - row + c * stride + D / 4 * BM) + row);
-      };
-      // O = sum_c 2^(m_c - M) O_c / sum_c 2^(m_c - M) l_c, M = max_c m_c (a split launch is
-      // never block-masked: every m_c is finite)
-      // up to kMergeAhead loads per thread in flight: a merge is a chain of L2 round trips
-      constexpr int kMergeAhead = 4;
-      float M = -INFINITY, L = 0.f;
-      for (int c0 = 0; c0 < sc.C; c0 += kMergeAhead) {
-        float2 v[kMergeAhead];
-#pragma unroll
-        for (int i = 0; i < kMergeAhead; ++i) v[i] = ml(min(c0 + i, sc.C - 1));
-        float m_new = M;
-#pragma unroll
-        for (int i = 0; i < kMergeAhead; ++i) m_new = fmaxf(m_new, v[i].x);
-        L *= ex2_approx(M - m_new);
-        M = m_new;
-#pragma unroll
-        for (int i = 0; i < kMergeAhead; ++i)
-          if (c0 + i < sc.C) L += v[i].y * ex2_approx(v[i].x - M);
-      }
-      const float inv_L = 1.0f / L;
-      float acc[32];
-      auto add = [&](float wgt, const float4(&v)[8]) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          acc[4 * q] = fmaf(v[q].x, wgt, acc[4 * q]);
-          acc[4 * q + 1] = fmaf(v[q].y, wgt, acc[4 * q + 1]);
-          acc[4 * q + 2] = fmaf(v[q].z, wgt, acc[4 * q + 2]);
-          acc[4 * q + 3] = fmaf(v[q].w, wgt, acc[4 * q + 3]);
-        }
-      };
-      // two blocks of 32 columns at a time, each with two ranges, or one block with
-      // kMergeAhead ranges at a time
-      const int blocks = sc.C <= 2 ? 2 : 1, at_once = kMergeAhead / blocks;
-#pragma unroll 1
-      for (int cc = 0; cc < D / 32; cc += blocks) {
-#pragma unroll
-        for (int e = 0; e < 32; ++e) acc[e] = 0.f;
-#pragma unroll 1
-        for (int c0 = 0; c0 < sc.C; c0 += at_once) {
-          float4 v[kMergeAhead][8];
-          float m_c[kMergeAhead];
-#pragma unroll
-          for (int i = 0; i < kMergeAhead; ++i) {
-            const int blk = blocks == 2 ? i / 2 : 0;
-            const int c = min(c0 + (blocks == 2 ? i % 2 : i), sc.C - 1);
-            m_c[i] = ml(c).x;
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-              v[i][q] = __ldcg(base + c * stride + ((cc + blk) * 8 + q) * BM);
-          }
-#pragma unroll
-          for (int i = 0; i < kMergeAhead; ++i) {
-            if (blocks == 2 && i == 2) {
-              if (valid) store_row_bf16<32>(orow + cc * 32, acc, inv_L);
-#pragma unroll
-              for (int e = 0; e < 32; ++e) acc[e] = 0.f;
-            }
-            if (c0 + (blocks == 2 ? i % 2 : i) < sc.C) add(ex2_approx(m_c[i] - M), v[i]);
-          }
-        }
-        if (valid) store_row_bf16<32>(orow + (cc + blocks - 1) * 32, acc, inv_L);
-      }
-      if (valid && p.lse)
-        p.lse[static_cast<int64_t>(u.h) * p.S_tok + token] =
-            (M + __log2f(L)) * 0.69314718055994531f;
-    }
-    if (row == 0) p.ws_count[2 * u.item + X] = 0;  // ready for the next launch
   }
   return true;
 }
@@ -1123,8 +1223,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   volatile int* mma_done = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 24);  // [2]
   const int warp = threadIdx.x >> 5;
 
-  // the schedule's only input is read while the barriers and TMEM are set up
-  const Sched sc = make_sched(p);
+  // in shared memory: the roles look at it between units, and it would cost the softmax loop
+  // registers
+  __shared__ Sched sc;
+  if (threadIdx.x == 64) sc = make_sched(p);
   if (threadIdx.x == 0) {
     for (int X = 0; X < 2; ++X) {
       mbar_init(bar0 + 8 * (C::kBarQFull + X), 1);
@@ -1377,8 +1479,10 @@ rf_status make_map(CUtensorMap* m, const void* base, int d, int H, int S_tok, in
 // Block-masked launches (which never split) use counters 0 and 1 for the work queue, 2.. for
 // the longest-first pre-pass's groups, and the partial-row area for the items' costs and order.
 constexpr int64_t kCountBytes = kMaxGrid * 4;
-int64_t workspace_bytes(int d, int grid) {
-  return kCountBytes + static_cast<int64_t>(grid) * 2 * BM * (d + 4) * 4;
+// `slots` partial slots per CTA: with one, the tail's items can be split into equal ranges, with two
+// it can also be dealt out evenly.
+int64_t workspace_bytes(int d, int grid, int slots) {
+  return kCountBytes + static_cast<int64_t>(grid) * slots * 2 * BM * (d + 4) * 4;
 }
 
 template <int D, bool MASKED>
@@ -1400,11 +1504,11 @@ rf_status launch(const CUtensorMap& q, const CUtensorMap& q128, const CUtensorMa
 }
 
 // Scratch for rf_attn_noalloc: a file-scope device array, so that callers who cannot allocate
-// device memory still get split-KV.  Sized for head dim 128 on up to 160 SMs (20.6 MiB); every
+// device memory still get split-KV.  Sized for head dim 128 on up to 160 SMs (41.3 MiB); every
 // GPU that loads this library holds it until the process exits.
 constexpr int kNoAllocMaxGrid = 160;
 constexpr int64_t kNoAllocScratchBytes =
-    kCountBytes + static_cast<int64_t>(kNoAllocMaxGrid) * 2 * BM * (128 + 4) * 4;
+    kCountBytes + static_cast<int64_t>(kNoAllocMaxGrid) * 2 * 2 * BM * (128 + 4) * 4;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 std::mutex g_noalloc_mu;
 void* g_noalloc_addr[64] = {};  // device address of the array, per device ordinal
@@ -1419,7 +1523,7 @@ extern "C" int64_t rf_attn_workspace_bytes(int d) {
   DeviceInfo di;
   if (current_device_info(&di) != RF_OK) return -1;
   const int grid = di.sm_count < kMaxGrid ? di.sm_count : kMaxGrid;
-  return workspace_bytes(d, grid);
+  return workspace_bytes(d, grid, 2);
 }
 
 namespace {
@@ -1479,7 +1583,7 @@ rf_status attn_impl(void* d_O, float* d_lse, const void* d_Q, const void* d_K, c
   const int64_t tiles = (rows + BM - 1) / BM;
   const int64_t max_items = ((tiles + 1) / 2) * H;
   int grid = di.sm_count < kMaxGrid ? di.sm_count : kMaxGrid;
-  const bool split = d_workspace != nullptr && workspace_bytes_given >= workspace_bytes(d, grid);
+  const bool split = d_workspace != nullptr && workspace_bytes_given >= workspace_bytes(d, grid, 1);
   // without split-KV there is no use for more CTAs than items
   if (!split && max_items < grid) grid = static_cast<int>(max_items);
   if (grid < 1) grid = 1;
@@ -1493,6 +1597,7 @@ rf_status attn_impl(void* d_O, float* d_lse, const void* d_Q, const void* d_K, c
   p.ws_count = split ? static_cast<int*>(d_workspace) : nullptr;
   p.ws_part = split ? reinterpret_cast<float*>(static_cast<char*>(d_workspace) + kCountBytes)
                     : nullptr;
+  p.ws_slots = split && workspace_bytes_given >= workspace_bytes(d, grid, 2) ? 2 : 1;
   p.block_mask = d_block_mask;
   p.lpt_order = nullptr;
   p.lpt_bits = nullptr;
@@ -1515,12 +1620,12 @@ rf_status attn_impl(void* d_O, float* d_lse, const void* d_Q, const void* d_K, c
     const int64_t kv_head = 4 * S_tok * d;  // bytes of one head's K and V
     const int64_t heads_l2 = std::max<int64_t>(1, di.l2_bytes / 2 / kv_head);
     if (split && (H + heads_l2 - 1) / heads_l2 <= kMaxLptGroups &&
-        2 * max_items * 4 <= workspace_bytes(d, grid) - kCountBytes) {
+        2 * max_items * 4 <= workspace_bytes(d, grid, 1) - kCountBytes) {
       int* cost = reinterpret_cast<int*>(p.ws_part);
       int* order = cost + max_items;
       // the items' tile bitmaps after them, where there is room (else the CTAs scan the mask again)
       const int64_t words = (p.nkv + 31) / 32;
-      if ((2 + words) * max_items * 4 <= workspace_bytes(d, grid) - kCountBytes)
+      if ((2 + words) * max_items * 4 <= workspace_bytes(d, grid, 1) - kCountBytes)
         p.lpt_bits = reinterpret_cast<uint32_t*>(order + max_items);
       p.lpt_heads_l2 = static_cast<int>(std::min<int64_t>(heads_l2, H));
       p.lpt_grid = grid;

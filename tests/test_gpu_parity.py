@@ -620,6 +620,53 @@ def test_attn_split_and_unsplit_agree_with_oracle(cuda_lib, F, N, H, d, mask):
     assert (O1.float() - O2.float()).abs().max().item() < 1e-2
 
 
+@pytest.mark.parametrize("F,N,H,d,A", [
+    (13, 1560, 1, 128, 13),   # 80 items: the whole launch dealt evenly over 152 CTAs
+    (7, 1003, 5, 128, 5),     # 100 items, frames off the tile boundaries, a last key tile of 109
+    (13, 1560, 3, 128, 13),   # 240 items: one full round, then 88 items dealt evenly
+    (13, 1560, 1, 64, 8),     # 49 items at head dim 64
+    (3, 1024, 12, 128, 3),    # 144 items of 24 key tiles: too close to a full round
+    (5, 700, 8, 128, 5),      # 112 items
+])
+def test_attn_dealt_evenly(cuda_lib, F, N, H, d, A):
+    """A last round of more than a quarter as many items as CTAs is dealt out by key tiles, and an
+    item may be in pieces of different length on neighbouring CTAs.  With the full workspace,
+    with the smaller one that only splits into equal ranges, and without: every result within
+    tolerance of the oracle on rows of every tile pair, close to the others, and repeatable."""
+    rf = cuda_lib
+    Q, K, V = _qkv(F * N, H, d, seed=F * 31 + N + d)
+    mask = [0] * F
+    for i in range(A):
+        mask[i * F // A] = 1
+    scale = 1.0 / math.sqrt(d)
+    act, skp = (torch.zeros(F, dtype=torch.int32, device=DEV) for _ in range(2))
+    cnt = torch.zeros(2, dtype=torch.int32, device=DEV)
+    rf.rf_schedule_compact(torch.tensor(mask, dtype=torch.uint8, device=DEV), F, N, act, skp,
+                           None, cnt)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    full = rf.rf_attn_workspace_bytes(d)
+    rows = sorted(set(_active_rows(mask, N)[::97] + _active_rows(mask, N)[-130:]))
+    Oref, Lref = oracle.attention(Q.cpu(), K.cpu(), V.cpu(), rows, scale)
+    outs = []
+    for nbytes in (full, full, (full - 4096) // 2 + 4096, 0):
+        ws = torch.zeros(nbytes // 4, dtype=torch.int32, device=DEV) if nbytes else None
+        O = torch.full((F * N, H, d), SENTINEL, dtype=torch.bfloat16, device=DEV)
+        L = torch.full((H, F * N), SENTINEL, device=DEV)
+        for _ in range(2):  # the second call finds the workspace as the first left it
+            rf.rf_attn(O, L, Q, K, V, Q.stride(0), O.stride(0), F, N, H, d, act, cnt, scale, ws,
+                       status)
+        torch.cuda.synchronize()
+        assert status.item() == 0
+        if ws is not None:
+            assert int(ws[:1024].abs().sum()) == 0, "merge counters not reset"
+        compare(O.cpu().float()[rows].numpy(), Oref, L.cpu()[:, rows].numpy(), Lref, str(nbytes))
+        skipped = sorted(set(range(F * N)) - set(_active_rows(mask, N)))
+        assert (O[skipped].float() == SENTINEL).all() and (L[:, skipped] == SENTINEL).all()
+        outs.append(O)
+    assert torch.equal(outs[0], outs[1])
+    assert all((outs[0].float() - o.float()).abs().max().item() < 1e-2 for o in outs[2:])
+
+
 def _pipeline_against_device_path(F, N, H, d, E, plan_args, Q, K0, V0, vel, z0, scale, nsteps,
                                   depth):
     """The same steps on device-resident inputs (StepCore, fresh K/V rows written before each
