@@ -33,7 +33,9 @@
 //   2368  one issuing warp per tile, taking turns: a warp waits for its own P, K and V while the
 //         other warp's MMAs run, instead of behind them in one instruction stream
 //   2290  the turn taken before the wait for P, not after it
-// At 2290 the sustained rate of long launches is set by the power cap (1.67 GHz against 1.80 before).
+//   2216  no registers spilled around the softmax loop (the split epilogue out of line)
+// (head dim 64: 1984).  At this pace the rate of long launches is set by the power cap: 1.65 GHz
+// under load, against 1.80 before.
 // Without the turns the two chains fall into step: both softmaxes at once, then both GEMM pairs
 // (4,300 cycles).  Each S_X(j+1) is committed after PV_X(j) was issued, so the softmax warps that
 // wait for S_X(j+1) also know that O_X is no longer being written and may rescale it in place.
@@ -83,12 +85,12 @@ constexpr uint32_t kTmemCols = 512;
 // on the barriers it owes (release_mma) until the waiting MMA warp, which reads the abort flag
 // in every round of its loop, has left.  All counts are multiples of a warp, so surplus arrivals
 // complete a barrier exactly.
-constexpr int kPSplit = 64;  // 32, 64, 96, 128: 2338, 2368, 2510, 2757 cycles per step
+constexpr int kPSplit = 64;  // 32, 64, 96: 2379, 2216, 2395 cycles per step (2051, 1984, 2150)
 constexpr int kPThreads = 128 + 32;
 __device__ __forceinline__ int p_barrier(int X, int part) { return 1 + 2 * X + part; }
 // The two MMA warps take turns; a turn is passed on before the last kTurnAhead MMAs of a group, so
-// that the other warp's MMAs follow without a gap (head dim 128: 0, 1, 2, 3, 4 measured within 1%;
-// head dim 64: 2051, 2081, 2130, 2212, 2230 cycles per step).
+// that the other warp's MMAs follow without a gap (head dim 128: 0 to 4 within 1%; head dim 64,
+// when the choice was made: 2051, 2081, 2130, 2212, 2230 cycles per step for 0 to 4).
 template <int D>
 constexpr int kTurnAhead = D == 128 ? 2 : 0;
 __device__ __forceinline__ int turn_barrier(int X) { return 5 + X; }
@@ -160,7 +162,7 @@ struct Sched {
   int R, tiles, pairs;  // active rows (padded per frame), query tiles and tile pairs per head
   int T_full;           // items processed whole
   int C;                // KV ranges per item of the split tail (1: no split)
-  uint32_t even_q, even_r;  // the tail dealt out evenly: its KV tiles / CTAs and the remainder (0: not)
+  uint32_t even_q, even_r;  // tail dealt out evenly: its KV tiles / CTAs, the remainder (0: not)
   int units;            // T_full + tail items * C, or + 2 per CTA (some empty) when dealt evenly
 };
 
@@ -175,15 +177,15 @@ struct Unit {
 // chosen by the KV tiles that the busiest CTA then processes:
 //   whole        nkv
 //   C ranges     nkv / C + kSplitCost, C = CTAs / items: every item in equal ranges, one per CTA
-//   dealt evenly tail * nkv / CTAs + kEvenCost: every CTA takes the same share of the tail's KV tiles,
-//                which may end in one item and begin the next (needs two partial slots per CTA)
+//   dealt evenly tail * nkv / CTAs + kEvenCost: every CTA takes the same share of the tail's KV
+//                tiles, which may end in one item and begin the next (two partial slots per CTA)
 // The costs are the boundary of a further unit and the merge, in KV tiles (dealt evenly, the
-// partials of all items are written and read: 34 MB each way for 100 items on 152 CTAs, some 10 us).
+// partials of all items are written and read: 34 MB each way for 100 items on 152 CTAs, 10 us).
 // Dealing evenly is considered where C ranges leave CTAs idle: more than a quarter as many items as
 // CTAs (below, the items' ranges fill the chip and an item would be in more than five pieces).
 // Measured (us per launch, whole or in C ranges -> dealt evenly): 13 x 1560 tokens x 1 head x 128
-// (80 items) 186 -> 122; 9 of the 13 frames active (55 items) 107 -> 93; 7 x 1003 x 5 x 128, 5 active
-// (100 items of 55 tiles) 70.3 -> 66.9.
+// (80 items) 186 -> 122; 9 of the 13 frames active (55 items) 107 -> 93; 7 x 1003 x 5 x 128, 5
+// active (100 items of 55 tiles) 70.3 -> 66.9.
 constexpr int kSplitCost = 3, kEvenCost = 10;
 constexpr uint32_t kMinEvenShare = 12;  // KV tiles per CTA
 // KV tile, counted over the whole tail, where CTA k's share begins; no piece is shorter than
