@@ -206,18 +206,18 @@ def run_gpu(args):
         t0.record(stream)
         for k in range(K_steps):
             s = k % S
-            c.compact(s)
+            if not per_launch:
+                c.run(s, vel[s], O, Q, K, V, w.softmax_scale)
+                continue
+            c.compact(s)  # the step's parts call by call, to time the attention launch alone
             c.project(s)
             c.project_kv(s, K, V)
-            if per_launch:
-                a = torch.cuda.Event(enable_timing=True)
-                b = torch.cuda.Event(enable_timing=True)
-                a.record(stream)
-                c.attn(O, Q, K, V, w.softmax_scale)
-                b.record(stream)
-                ev.append((s, a, b))
-            else:
-                c.attn(O, Q, K, V, w.softmax_scale)
+            a = torch.cuda.Event(enable_timing=True)
+            b = torch.cuda.Event(enable_timing=True)
+            a.record(stream)
+            c.attn(O, Q, K, V, w.softmax_scale)
+            b.record(stream)
+            ev.append((s, a, b))
             c.step(s, vel[s])
         t1.record(stream)
         barrier()
@@ -241,7 +241,7 @@ def run_gpu(args):
     per_launch_flops = attn_flops_total / len(ev)
     # all-frames-active comparison, same number of steps
     ms_all, _ = timed(core_all, K_steps, min(W_steps, 3))
-    # the step core's five launches, each timed on its own over one trajectory (the latent-width
+    # the step's five parts, each launched and timed on its own over one trajectory (the latent-width
     # kernels are launch-bound, so their microseconds are reported, not GB/s)
     parts = {"rf_schedule_compact": [], "rf_project": [], "rf_project_kv": [], "rf_attn": [],
              "rf_step": []}

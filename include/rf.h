@@ -9,7 +9,7 @@
  * linear projection of their latent trajectory (Eq. 3).  Afterwards only the
  * active frames take their Euler step.
  *
- * One step of that core is five calls, all asynchronous on a caller-provided
+ * One step of that core is five calls (or rf_step_core), all asynchronous on a caller-provided
  * CUDA stream and all working on caller-owned device buffers:
  *
  *   rf_schedule_compact  active-frame mask -> frame / token index lists
@@ -289,6 +289,24 @@ rf_status rf_attn_noalloc(void* d_O, float* d_lse, const void* d_Q, const void* 
 rf_status rf_step(float* d_z2, const uint8_t* d_cur_slot, const float* d_v, const float* d_dt,
                   const int32_t* d_active, const int32_t* d_counts, int F, int64_t E,
                   rf_stream_t stream);
+
+/*
+ * rf_step_core -- a whole step: rf_schedule_compact, rf_project, rf_project_kv (if d_Kc and d_Vc
+ * are given; both NULL: without the cache), rf_attn and rf_step, with the arguments of those
+ * calls and D = H*d.  Every argument is checked before anything is enqueued; the first error, in
+ * that order, is returned.  Same results as the five calls, in two launches: everything but the
+ * attention shares one.  Where the buffers overlap in a way that needs the calls' order (d_v a
+ * view of d_ctx or of d_O, say), each part is launched by itself in that order.
+ *   qkv_row_stride  of d_Q, d_K, d_V in the attention; kv_row_stride of d_K, d_V in the cache step
+ */
+rf_status rf_step_core(const uint8_t* d_mask, const uint8_t* d_cur_slot, const float* d_alpha,
+                       const float* d_beta, const float* d_dt, int F, int N, int64_t E, int H,
+                       int d, int32_t* d_active, int32_t* d_skipped, int32_t* d_token_idx,
+                       int32_t* d_counts, float* d_ctx, float* d_z2, const float* d_v, void* d_Kc,
+                       void* d_Vc, void* d_O, float* d_lse, const void* d_Q, void* d_K, void* d_V,
+                       int64_t qkv_row_stride, int64_t kv_row_stride, int64_t o_row_stride,
+                       float softmax_scale, void* d_workspace, int64_t workspace_bytes,
+                       int32_t* d_status, rf_stream_t stream);
 
 /*
  * rf_frame_gram -- inner products of the F clean-latent proxies, the input of sequential

@@ -16,7 +16,7 @@ import numpy as np
 
 __all__ = ["load", "lib_path", "RFError", "rf_plan_build", "rf_schedule_compact",
            "rf_project", "rf_project_kv", "rf_attn", "rf_attn_block_masked",
-           "rf_attn_workspace_bytes", "rf_attn_noalloc", "rf_step", "rf_frame_gram",
+           "rf_attn_workspace_bytes", "rf_attn_noalloc", "rf_step", "rf_step_core", "rf_frame_gram",
            "rf_keyframe_select", "rf_selftest_bounded_wait", "rf_pipeline_create",
            "rf_pipeline_step", "rf_pipeline_sync", "rf_pipeline_bytes", "rf_pipeline_destroy",
            "rf_status_str", "rf_version", "EXPORTS"]
@@ -28,7 +28,7 @@ _LIB: Optional[ctypes.CDLL] = None
 EXPORTS = ("rf_status_str", "rf_version", "rf_last_error", "rf_plan_build",
            "rf_schedule_compact", "rf_project", "rf_project_kv", "rf_attn",
            "rf_attn_block_masked", "rf_attn_workspace_bytes",
-           "rf_attn_noalloc", "rf_step", "rf_frame_gram", "rf_keyframe_select",
+           "rf_attn_noalloc", "rf_step", "rf_step_core", "rf_frame_gram", "rf_keyframe_select",
            "rf_pipeline_create", "rf_pipeline_step", "rf_pipeline_sync", "rf_pipeline_bytes",
            "rf_pipeline_destroy", "rf_selftest_bounded_wait")
 
@@ -54,6 +54,8 @@ _SIG = {
     "rf_attn_noalloc": ([_vp, _vp, _vp, _vp, _vp, _i64, _i64, _i32, _i32, _i32, _i32, _vp, _vp,
                          _f32, _vp, _vp], _i32),
     "rf_step": ([_vp, _vp, _vp, _vp, _vp, _vp, _i32, _i64, _vp], _i32),
+    "rf_step_core": ([_vp] * 5 + [_i32, _i32, _i64, _i32, _i32] + [_vp] * 14 +
+                     [_i64, _i64, _i64, _f32, _vp, _i64, _vp, _vp], _i32),
     "rf_pipeline_create": ([_i32, _i32, _i32, _i32, _i64, _i32, _vp, _vp, _vp, _vp, _vp, _vp,
                             _vp, _vp, _i32, _vp, _vp, _vp, ctypes.POINTER(_vp)], _i32),
     "rf_pipeline_step": ([_vp, _i32, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _f32], _i32),
@@ -222,6 +224,20 @@ def rf_step(z2, cur_slot, v, dt, active, counts, F: int, E: int, stream=None):
     _check("rf_step", load().rf_step(
         _ptr(z2), _ptr(cur_slot), _ptr(v), _ptr(dt), _ptr(active), _ptr(counts), F, E,
         _stream(stream)))
+
+
+def rf_step_core(mask, cur_slot, alpha, beta, dt, F: int, N: int, E: int, H: int, d: int, active,
+                 skipped, token_idx, counts, ctx, z2, v, Kc, Vc, O, lse, Q, K, V,
+                 qkv_row_stride: int, kv_row_stride: int, o_row_stride: int,
+                 softmax_scale: float, workspace=None, status=None, stream=None):
+    """A whole step in two launches; Kc and Vc None: without the rolling cache."""
+    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
+    _check("rf_step_core", load().rf_step_core(
+        _ptr(mask), _ptr(cur_slot), _ptr(alpha), _ptr(beta), _ptr(dt), F, N, E, H, d,
+        _ptr(active), _ptr(skipped), _ptr(token_idx), _ptr(counts), _ptr(ctx), _ptr(z2), _ptr(v),
+        _ptr(Kc), _ptr(Vc), _ptr(O), _ptr(lse), _ptr(Q), _ptr(K), _ptr(V), qkv_row_stride,
+        kv_row_stride, o_row_stride, float(softmax_scale), _ptr(workspace), ws_bytes,
+        _ptr(status), _stream(stream)))
 
 
 def rf_pipeline_create(F: int, N: int, H: int, d: int, E: int, plan: dict, z2, K0, V0,

@@ -1645,6 +1645,17 @@ rf_status attn_impl(void* d_O, float* d_lse, const void* d_Q, const void* d_K, c
 }
 }  // namespace
 
+rf_status rf::attn_check(const void* d_O, const void* d_Q, const void* d_K, const void* d_V,
+                         int64_t qkv_row_stride, int64_t o_row_stride, int F, int N, int H,
+                         int d, const int32_t* d_active, const int32_t* d_counts,
+                         float softmax_scale, const void* d_workspace,
+                         int64_t workspace_bytes_given) {
+  DeviceInfo di;
+  return check_attn_args(d_O, d_Q, d_K, d_V, qkv_row_stride, o_row_stride, F, N, H, d, d_active,
+                         d_counts, softmax_scale, nullptr, d_workspace, workspace_bytes_given,
+                         &di);
+}
+
 extern "C" rf_status rf_attn(void* d_O, float* d_lse, const void* d_Q, const void* d_K,
                              const void* d_V, int64_t qkv_row_stride, int64_t o_row_stride, int F,
                              int N, int H, int d, const int32_t* d_active,

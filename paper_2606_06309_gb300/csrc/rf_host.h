@@ -30,4 +30,10 @@ inline rf_status launch_status(const char* what) {
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// The argument errors of rf_attn, with nothing enqueued.
+rf_status attn_check(const void* d_O, const void* d_Q, const void* d_K, const void* d_V,
+                     int64_t qkv_row_stride, int64_t o_row_stride, int F, int N, int H, int d,
+                     const int32_t* d_active, const int32_t* d_counts, float softmax_scale,
+                     const void* d_workspace, int64_t workspace_bytes);
+
 }  // namespace rf

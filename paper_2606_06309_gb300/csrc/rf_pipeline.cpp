@@ -231,15 +231,11 @@ extern "C" rf_status rf_pipeline_step(rf_pipeline* p, int s, const void* h_Q, co
     CUDA_TRY(cudaStreamWaitEvent(p->compute, B.drained, 0), "rf_pipeline compute wait");
   const rf_stream_t cs = reinterpret_cast<rf_stream_t>(p->compute);
   const size_t o = static_cast<size_t>(s) * F;
-  RF_TRY(rf_schedule_compact(p->mask + o, F, p->N, p->active, p->skipped, nullptr, p->counts, cs));
-  RF_TRY(rf_project(p->ctx, p->z2, p->cur_slot + o, p->alpha + o, p->beta + o, F, p->E, cs));
   const int64_t hd = static_cast<int64_t>(p->H) * p->d;
-  // skipped frames' keys and values: Eq. 3 over the cache; active frames' fresh rows shifted in
-  RF_TRY(rf_project_kv(B.K, B.V, hd, p->Kc, p->Vc, p->cur_slot + o, p->alpha + o, p->beta + o,
-                       p->active, p->skipped, p->counts, F, p->N, static_cast<int>(hd), cs));
-  RF_TRY(rf_attn(B.O, nullptr, B.Q, B.K, B.V, hd, hd, F, p->N, p->H, p->d, p->active, p->counts,
-                 softmax_scale, p->ws, p->ws_bytes, p->status, cs));
-  RF_TRY(rf_step(p->z2, p->cur_slot + o, B.v, p->dt + o, p->active, p->counts, F, p->E, cs));
+  RF_TRY(rf_step_core(p->mask + o, p->cur_slot + o, p->alpha + o, p->beta + o, p->dt + o, F, p->N,
+                      p->E, p->H, p->d, p->active, p->skipped, nullptr, p->counts, p->ctx, p->z2,
+                      B.v, p->Kc, p->Vc, B.O, nullptr, B.Q, B.K, B.V, hd, hd, hd, softmax_scale,
+                      p->ws, p->ws_bytes, p->status, cs));
   CUDA_TRY(cudaMemcpyAsync(B.z, p->z2, 2 * FE4, cudaMemcpyDeviceToDevice, p->compute),
            "rf_pipeline state snapshot");
   if (h_ctx)

@@ -951,6 +951,78 @@ def test_graph_replay_matches_eager(cuda_lib, name):
     assert cg.status.item() == 0
 
 
+# F past one 128-frame tile of the mask, token chunks of 2048, latent and K/V chunks of 512
+# vectors: sizes at and beside the edges
+@pytest.mark.parametrize("F,N,C,H,d,every,fused", [
+    (1, 1, 4, 1, 64, 1, False), (4, 64, 16, 2, 64, 3, False), (5, 2049, 4, 1, 64, 2, True),
+    (33, 130, 16, 3, 128, 5, True), (129, 9, 8, 1, 64, 4, False), (300, 16, 4, 1, 128, 7, False),
+    (3, 512, 4, 2, 64, 99, False),
+])
+@pytest.mark.parametrize("cache,tokens", [(True, True), (False, False)])
+def test_step_core_matches_the_five_calls(cuda_lib, F, N, C, H, d, every, fused, cache, tokens):
+    """run() (all but the attention in one launch) gives, bit for bit, what the five calls give:
+    active frames whose context reads both slots (a plan made by hand), skipped frames with
+    beta == 0, no active frame at all (every = 99 with frame 0 off), K and V rows of a fused
+    buffer, and a velocity that is a view of the context (parts launched in order)."""
+    from paper_2606_06309_gb300.stepcore import Plan, StepCore
+    g = torch.Generator().manual_seed(F * 1000 + N)
+    E = N * C
+    mask = torch.tensor([[1 if every < 99 and f % every == 0 else 0 for f in range(F)]] * 2,
+                        dtype=torch.uint8)
+    beta = torch.rand(2, F, generator=g)
+    beta[0, ::2] = 0.0
+    t = {"mask": mask, "alpha": 1.0 - beta, "beta": beta, "dt": torch.rand(2, F, generator=g),
+         "cur_slot": torch.randint(0, 2, (2, F), generator=g, dtype=torch.uint8)}
+    plan = Plan(*(t[k].to(DEV) for k in ("mask", "alpha", "beta", "dt", "cur_slot")), {})
+    z = torch.randn(2, F, E, generator=g).to(DEV)
+    v = torch.randn(F, E, generator=g).to(DEV)
+    rows = torch.randn(F * N, 3, H, d, generator=g).to(DEV, torch.bfloat16)
+    c0 = torch.randn(2, 2, F, N, H * d, generator=g).to(DEV, torch.bfloat16)
+
+    def case(together, v_is_ctx):
+        core = StepCore(F, N, E, H, d, plan, DEV, token_list=tokens, kv_cache=cache)
+        core.z2.copy_(z)
+        if cache:
+            core.Kc.copy_(c0[0])
+            core.Vc.copy_(c0[1])
+        b = rows.clone()
+        Q, K, V = ((b[:, i] if fused else b[:, i].contiguous()) for i in range(3))
+        O = torch.zeros(F * N, H, d, dtype=torch.bfloat16, device=DEV)
+        vel = core.ctx if v_is_ctx else v
+        for s in range(2):
+            if together:
+                core.run(s, vel, O, Q, K, V, 0.1)
+            else:
+                core.compact(s)
+                core.project(s)
+                if cache:
+                    core.project_kv(s, K, V)
+                core.attn(O, Q, K, V, 0.1)
+                core.step(s, vel)
+        assert core.status.item() == 0
+        return [core.active, core.skipped, core.token_idx, core.counts, core.ctx, core.z2,
+                core.Kc, core.Vc, K, V, O]
+
+    for v_is_ctx in (False, True):
+        for a, b in zip(case(True, v_is_ctx), case(False, v_is_ctx)):
+            assert (a is None and b is None) or torch.equal(a, b)
+
+
+def test_step_core_errors_are_those_of_the_call_at_fault(cuda_lib):
+    """A refused argument: the same error as from the five calls, and the latent store as it was."""
+    from paper_2606_06309_gb300.stepcore import StepCore, upload_plan
+    F, N, H, d = 4, 64, 2, 64
+    core = StepCore(F, N, N * 4, H, d, upload_plan(F, 2, [1] * F, [1, 1], 0, DEV), DEV)
+    core.set_state(torch.ones(F, N * 4, device=DEV))
+    x = torch.zeros(F * N, H, d, dtype=torch.bfloat16, device=DEV)
+    v = torch.zeros(F * N * 4 + 1, device=DEV)
+    with pytest.raises(cuda_lib.RFError, match="rf_attn failed"):
+        core.run(0, v[:-1], x, x.clone(), x.clone(), x.clone(), -1.0)
+    with pytest.raises(cuda_lib.RFError, match="rf_step failed"):
+        core.run(0, v[1:], x, x.clone(), x.clone(), x.clone(), 0.1)
+    assert torch.equal(core.z2, torch.ones_like(core.z2))
+
+
 # ---------------------------------------------------------------------------
 # rf_attn_block_masked: frame mask x token block mask (Appendix D)
 # ---------------------------------------------------------------------------
