@@ -6,7 +6,8 @@
 // once (the Gram matrix; its diagonal gives the norms) and the host runs the sequential rule
 // over it (rf_keyframe_select in rf_plan.cpp).
 //
-// Kernel: split-K over the proxy length E.  Each CTA takes every n-th slice of up to 128
+// gram_kernel (gram_short_kernel below some ten thousand elements, see gram_long_from): split-K
+// over the proxy length E.  Each CTA takes every n-th slice of up to 128
 // elements of every frame, streams them through shared memory (cp.async, two or three stages,
 // rows as they are in memory) and accumulates 8 x 8 frame pairs per thread in fp32, four
 // elements at a time.  Only tiles on and above the diagonal have threads: with G = ceil(F/8)
@@ -206,12 +207,134 @@ __global__ void __launch_bounds__(kGramThreads, 2)
     const int a = (e / T) % T, b = e % T;
     const int fi = ti + a * groups, fj = tj + b * groups;
     if (fi < F && fj < F && (ti != tj || a <= b)) {
-      const double t = static_cast<double>(hi) + static_cast<double>(lo);
+      // an infinite or undefined sum is in hi; the rounding errors beside it are not numbers
+      const double t = isfinite(hi) ? static_cast<double>(hi) + static_cast<double>(lo)
+                                    : static_cast<double>(hi);
       atomicAdd(out + static_cast<int64_t>(fi) * F + fj, t);
       if (fi != fj) atomicAdd(out + static_cast<int64_t>(fj) * F + fi, t);
     }
   }
   cluster.sync();  // no CTA leaves while another reads its shared memory
+}
+
+// Short proxies: a grid of plain CTAs, each 128 elements of every frame (or a few such slices), TILE
+// frames (>= F, padded with zeros).  Thread tiles are 4 x 4; (TILE/4)^2 threads form a
+// k-group, and the 256/((TILE/4)^2) k-groups of a CTA take interleaved elements of each stage,
+// so small F does not pay for a 64 x 64 product.  The Gram matrix is symmetric: thread tiles
+// below the diagonal are skipped and the upper ones written to both halves.  The next stage's
+// global loads are issued before the current stage is multiplied (register double buffer).
+template <int TILE>
+__global__ void __launch_bounds__(kGramThreads)
+    gram_short_kernel(const float* __restrict__ P, int F, int64_t E, int64_t ld, double* __restrict__ G) {
+  constexpr int TG = (TILE / 4) * (TILE / 4);  // threads per k-group
+  static_assert(TILE % 8 == 0 && TG <= kGramThreads && kGramK % 16 == 0, "tile");
+  constexpr int KG = kGramThreads / TG;          // k-groups per CTA (leftover threads only load)
+  constexpr int kStageV = TILE * kGramK / 4;     // float4 per stage
+  constexpr int NV = (kStageV + kGramThreads - 1) / kGramThreads;  // per thread
+  __shared__ __align__(16) float tile[kGramK][TILE + 4];
+  __shared__ float red[KG > 1 ? KG : 1][TG][16];
+  const int g = threadIdx.x / TG, r = threadIdx.x % TG;
+  const int ty = r / (TILE / 4), tx = r % (TILE / 4);
+  const bool upper = g < KG && ty <= tx;
+  float acc[4][4] = {};
+  const bool vec_ok = (ld % 4 == 0) && ((reinterpret_cast<uintptr_t>(P) & 15) == 0);
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * kGramK;
+  float4 pre[NV];
+  // float4 v of a stage -> (frame lf, element lk): a warp's 32 consecutive v cover 8 frames x 16
+  // elements (64 contiguous bytes per frame), so the transposed stores below spread over 16
+  // banks (2-way) where 32 rows of one frame column would fall into 2 banks (16-way)
+  auto frame_of = [](int v) { return ((v >> 5) % (TILE / 8)) * 8 + ((v & 31) >> 2); };
+  auto elem_of = [](int v) { return ((v >> 5) / (TILE / 8)) * 16 + (v & 3) * 4; };
+  auto load = [&](int64_t k0) {
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      const int v = threadIdx.x + q * kGramThreads;
+      const int idx = v * 4;
+      const int lf = frame_of(v), lk = elem_of(v);
+      const float* prow = P + static_cast<int64_t>(lf) * ld + k0 + lk;
+      if (idx >= kStageV * 4) {
+        pre[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+      } else if (lf < F && vec_ok && k0 + lk + 4 <= E) {
+        pre[q] = __ldcs(reinterpret_cast<const float4*>(prow));
+      } else {
+        float t[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) t[e] = (lf < F && k0 + lk + e < E) ? prow[e] : 0.f;
+        pre[q] = make_float4(t[0], t[1], t[2], t[3]);
+      }
+    }
+  };
+  int64_t k0 = static_cast<int64_t>(blockIdx.x) * kGramK;
+  if (k0 < E) load(k0);
+  for (; k0 < E; k0 += stride) {
+    __syncthreads();  // the previous stage has been consumed
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      const int v = threadIdx.x + q * kGramThreads;
+      if (v * 4 >= kStageV * 4) break;
+      const int lf = frame_of(v), lk = elem_of(v);
+      tile[lk][lf] = pre[q].x;
+      tile[lk + 1][lf] = pre[q].y;
+      tile[lk + 2][lf] = pre[q].z;
+      tile[lk + 3][lf] = pre[q].w;
+    }
+    __syncthreads();
+    if (k0 + stride < E) load(k0 + stride);  // in flight while this stage is multiplied
+    if (upper) {
+#pragma unroll 4
+      for (int k = g; k < kGramK; k += KG) {
+        const float4 a = *reinterpret_cast<const float4*>(&tile[k][ty * 4]);
+        const float4 b = *reinterpret_cast<const float4*>(&tile[k][tx * 4]);
+        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int jj = 0; jj < 4; ++jj) acc[i][jj] = fmaf(av[i], bv[jj], acc[i][jj]);
+      }
+    }
+  }
+  if (KG > 1) {  // sum the k-groups' partial tiles
+    if (g < KG) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) red[g][r][i * 4 + jj] = acc[i][jj];
+    }
+    __syncthreads();
+    if (g != 0) return;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int jj = 0; jj < 4; ++jj) {
+        float t = 0.f;
+        for (int q = 0; q < KG; ++q) t += red[q][r][i * 4 + jj];
+        acc[i][jj] = t;
+      }
+  }
+  if (!upper) return;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj) {
+      const int fi = ty * 4 + i, fj = tx * 4 + jj;
+      if (fi < F && fj < F && acc[i][jj] != 0.f && (ty < tx || fi <= fj)) {
+        atomicAdd(G + static_cast<int64_t>(fi) * F + fj, static_cast<double>(acc[i][jj]));
+        if (fi != fj)
+          atomicAdd(G + static_cast<int64_t>(fj) * F + fi, static_cast<double>(acc[i][jj]));
+      }
+    }
+}
+
+// Elements from which gram_kernel is the faster: below, its clusters, its wider tiles' fewer
+// threads and its sums cost more than one atomic per entry and CTA.  Short / long, in us:
+// 1 x 24000 7.3 / 8.4, 46000 8.4 / 8.3; 13 x 10001 8.4 / 10.4, 24960 14.4 / 10.4; 33 x 12000 9.9 / 12.5,
+// 24000 14.2 / 13.0, 27001 14.7 / 14.4, 57600 26.0 / 15.2; 56 x 20000 16.3 / 16.7, 30000 18.2 / 17.1;
+// 64 x 2475 10.0 / 27.5, 30000 18.9 / 23.5, 42000 28.4 / 24.3.
+int64_t gram_long_from(int F, bool vec) {
+  if (F <= 2 || (F > 56 && !vec)) return 40960;
+  if (F > 56) return 36864;  // two stages and 144 threads: 36 tiles leave no room for more k-groups
+  if (!vec && F > 16) return 30720;  // 4-byte copies into shared memory
+  return F > 48 ? 24576 : 20480;
 }
 
 }  // namespace
@@ -228,6 +351,23 @@ extern "C" rf_status rf_frame_gram(const float* d_P, int F, int64_t E, int64_t l
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (cudaError_t e = cudaMemsetAsync(d_G, 0, sizeof(double) * F * F, s))
     return fail(RF_ERR_CUDA, "cudaMemsetAsync(gram)", e);
+  const bool vec = ld % 4 == 0 && aligned16(d_P);
+  if (E < gram_long_from(F, vec)) {
+    int64_t blocks = (E + kGramK - 1) / kGramK;
+    if (blocks > 4LL * di.sm_count) blocks = 4LL * di.sm_count;
+    const int b = static_cast<int>(blocks);
+    if (F <= 16)
+      gram_short_kernel<16><<<b, kGramThreads, 0, s>>>(d_P, F, E, ld, d_G);
+    else if (F <= 24)
+      gram_short_kernel<24><<<b, kGramThreads, 0, s>>>(d_P, F, E, ld, d_G);
+    else if (F <= 40)
+      gram_short_kernel<40><<<b, kGramThreads, 0, s>>>(d_P, F, E, ld, d_G);
+    else if (F <= 48)
+      gram_short_kernel<48><<<b, kGramThreads, 0, s>>>(d_P, F, E, ld, d_G);
+    else
+      gram_short_kernel<64><<<b, kGramThreads, 0, s>>>(d_P, F, E, ld, d_G);
+    return launch_status("gram_short_kernel launch");
+  }
   const int groups = (F + kGramT - 1) / kGramT, tiles = groups * (groups + 1) / 2;
   int kgroups = 1;
   while (kgroups < kGramK / 4 && 2 * kgroups * tiles <= kGramThreads) kgroups *= 2;
@@ -247,7 +387,6 @@ extern "C" rf_status rf_frame_gram(const float* d_P, int F, int64_t E, int64_t l
   ctas = (ctas + kGramCluster - 1) / kGramCluster * kGramCluster;
   const int width = static_cast<int>(
       std::min<int64_t>(kGramK, ((E + ctas - 1) / ctas + 3) / 4 * 4));  // starts stay 16-byte aligned
-  const bool vec = ld % 4 == 0 && aligned16(d_P);
   const bool three = gram_stages(groups) == 3;
   auto kernel = vec ? (three ? gram_kernel<true, 3> : gram_kernel<true, 2>)
                     : (three ? gram_kernel<false, 3> : gram_kernel<false, 2>);
