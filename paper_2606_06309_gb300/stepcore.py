@@ -140,7 +140,8 @@ class StepCore:
             rf_step_core(_row(p.mask, s), _row(p.cur_slot, s), _row(p.alpha, s), _row(p.beta, s),
                          _row(p.dt, s), self.F, self.N, self.E, self.H, self.d, self.active,
                          self.skipped, self.token_idx, self.counts, self.ctx, self.z2, v, self.Kc,
-                         self.Vc, O, lse, Q, K, V, Q.stride(0), K.stride(0), O.stride(0), scale,
+                         self.Vc, O, lse, Q, K, V, Q.stride(0),
+                         0 if self.Kc is None else K.stride(0), O.stride(0), scale,
                          self.workspace, self.status, stream)
             return
         except RFError:

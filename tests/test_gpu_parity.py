@@ -868,7 +868,9 @@ def test_frame_gram_matches_fp64_matmul(cuda_lib, F, E, ld):
 
 @pytest.mark.parametrize("F", [1, 8, 9, 16, 17, 40, 41, 48, 64])
 @pytest.mark.parametrize("E,pad,shift", [(1, 0, 0), (127, 1, 0), (129, 3, 1), (3071, 1, 0),
-                                         (57600 + 5, 3, 0), (117000, 0, 1)])
+                                         (20479, 1, 0), (20480, 0, 0), (24575, 1, 0),
+                                         (36864, 0, 0), (40961, 2, 0), (57600 + 5, 3, 0),
+                                         (117000, 0, 1)])
 def test_frame_gram_tile_and_slice_edges(cuda_lib, F, E, pad, shift):
     """Frame groups of 8, slices cut short, rows and bases off the 16-byte boundaries.  Each fp32
     chain has at most 512 products (a CTA's elements over its k-groups), the rest is summed
@@ -884,6 +886,23 @@ def test_frame_gram_tile_and_slice_edges(cuda_lib, F, E, pad, shift):
     bound = 512 * 2.0 ** -24 * (p.abs() @ p.abs().t())
     assert ((G - p @ p.t()).abs() <= bound).all()
     assert torch.equal(G, G.t())
+
+
+@pytest.mark.parametrize("F,E", [(9, 300), (33, 57600), (64, 3000), (64, 60000)])
+def test_frame_gram_infinities_and_nan(cuda_lib, F, E):
+    """Products of an infinite or undefined element give what they give in 64 bits, and the other
+    entries stay numbers."""
+    rf = cuda_lib
+    P = torch.randn(F, E, generator=torch.Generator(device=DEV).manual_seed(E), device=DEV)
+    P[1, E // 2] = float("inf")
+    P[3, 5] = float("-inf")
+    P[6, E - 1] = float("nan")
+    G = torch.empty(F, F, dtype=torch.float64, device=DEV)
+    rf.rf_frame_gram(P, G)
+    want = P.double() @ P.double().t()
+    assert torch.equal(G.isnan(), want.isnan())
+    assert torch.equal(G.isinf(), want.isinf())
+    assert torch.equal(G[want.isinf()], want[want.isinf()])
 
 
 def test_keyframes_from_device_gram_match_oracle(cuda_lib):
@@ -990,8 +1009,9 @@ def test_step_core_matches_the_five_calls(cuda_lib, F, N, C, H, d, every, fused,
         O = torch.zeros(F * N, H, d, dtype=torch.bfloat16, device=DEV)
         vel = core.ctx if v_is_ctx else v
         for s in range(2):
-            if together:
-                core.run(s, vel, O, Q, K, V, 0.1)
+            if together:  # without the cache, keys and values may be plain addresses
+                core.run(s, vel, O, Q, K if cache else K.data_ptr(),
+                         V if cache else V.data_ptr(), 0.1)
             else:
                 core.compact(s)
                 core.project(s)
