@@ -6,7 +6,7 @@
 // once (the Gram matrix; its diagonal gives the norms) and the host runs the sequential rule
 // over it (rf_keyframe_select in rf_plan.cpp).
 //
-// gram_kernel (gram_short_kernel below some ten thousand elements, see gram_long_from): split-K
+// gram_kernel (gram_short_kernel where that is faster, see short_is_faster): split-K
 // over the proxy length E.  Each CTA takes every n-th slice of up to 128
 // elements of every frame, streams them through shared memory (cp.async, two or three stages,
 // rows as they are in memory) and accumulates 8 x 8 frame pairs per thread in fp32, four
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kGramThreads, 2)
   cluster.sync();  // no CTA leaves while another reads its shared memory
 }
 
-// Short proxies: a grid of plain CTAs, each 128 elements of every frame (or a few such slices), TILE
+// A grid of plain CTAs, each 128 elements of every frame (or a few such slices), TILE
 // frames (>= F, padded with zeros).  Thread tiles are 4 x 4; (TILE/4)^2 threads form a
 // k-group, and the 256/((TILE/4)^2) k-groups of a CTA take interleaved elements of each stage,
 // so small F does not pay for a 64 x 64 product.  The Gram matrix is symmetric: thread tiles
@@ -325,16 +325,25 @@ __global__ void __launch_bounds__(kGramThreads)
     }
 }
 
-// Elements from which gram_kernel is the faster: below, its clusters, its wider tiles' fewer
-// threads and its sums cost more than one atomic per entry and CTA.  Short / long, in us:
-// 1 x 24000 7.3 / 8.4, 46000 8.4 / 8.3; 13 x 10001 8.4 / 10.4, 24960 14.4 / 10.4; 33 x 12000 9.9 / 12.5,
-// 24000 14.2 / 13.0, 27001 14.7 / 14.4, 57600 26.0 / 15.2; 56 x 20000 16.3 / 16.7, 30000 18.2 / 17.1;
-// 64 x 2475 10.0 / 27.5, 30000 18.9 / 23.5, 42000 28.4 / 24.3.
-int64_t gram_long_from(int F, bool vec) {
-  if (F <= 2 || (F > 56 && !vec)) return 40960;
-  if (F > 56) return 36864;  // two stages and 144 threads: 36 tiles leave no room for more k-groups
-  if (!vec && F > 16) return 30720;  // 4-byte copies into shared memory
-  return F > 48 ? 24576 : 20480;
+// Whether gram_short_kernel is the faster of the two.  On short proxies gram_kernel's clusters, its
+// wider tiles' fewer threads and its sums cost more than one atomic per entry and CTA.  Short / long,
+// in us: 1 x 24000 7.3 / 8.4, 46000 8.4 / 8.3; 13 x 10001 8.4 / 10.4, 24960 14.4 / 10.4; 33 x 12000
+// 9.9 / 12.5, 24000 14.2 / 13.0, 27001 14.7 / 14.4, 57600 26.0 / 15.2; 56 x 20000 16.3 / 16.7, 30000
+// 18.2 / 17.1; 64 x 2475 10.0 / 27.5, 30000 18.9 / 23.5, 42000 28.4 / 24.3.
+// Long proxies whose rows are not 16-byte aligned go through 4-byte copies in gram_kernel, which
+// bound it where there is little arithmetic per element (9 to 24 frames) or few threads to issue
+// them (above 56): 16 x 1000001 49 / 44, 4000001 115 / 134; 21 x 2097153 110 / 113, 20 x 8000001 358 / 374;
+// 57 x 67483 37.8 / 39.0, 64 x 400001 118 / 105, 1000001 235 / 244.
+bool short_is_faster(int F, int64_t E, bool vec) {
+  int64_t long_from = F > 48 ? 24576 : 20480;
+  if (!vec && F > 16) long_from = F > 48 ? 32768 : 30720;
+  if (F > 56) long_from = vec ? 36864 : 73728;  // 36 tiles: 144 threads, two stages
+  if (F <= 2) long_from = 40960;
+  if (E < long_from) return true;
+  if (vec || F <= 8) return false;
+  if (F <= 16) return E >= 1572864;
+  if (F <= 24) return E >= 2097152;
+  return F > 56 && E >= 786432;
 }
 
 }  // namespace
@@ -352,7 +361,7 @@ extern "C" rf_status rf_frame_gram(const float* d_P, int F, int64_t E, int64_t l
   if (cudaError_t e = cudaMemsetAsync(d_G, 0, sizeof(double) * F * F, s))
     return fail(RF_ERR_CUDA, "cudaMemsetAsync(gram)", e);
   const bool vec = ld % 4 == 0 && aligned16(d_P);
-  if (E < gram_long_from(F, vec)) {
+  if (short_is_faster(F, E, vec)) {
     int64_t blocks = (E + kGramK - 1) / kGramK;
     if (blocks > 4LL * di.sm_count) blocks = 4LL * di.sm_count;
     const int b = static_cast<int>(blocks);

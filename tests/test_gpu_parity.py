@@ -874,7 +874,8 @@ def test_frame_gram_matches_fp64_matmul(cuda_lib, F, E, ld):
 def test_frame_gram_tile_and_slice_edges(cuda_lib, F, E, pad, shift):
     """Frame groups of 8, slices cut short, rows and bases off the 16-byte boundaries.  Each fp32
     chain has at most 512 products (a CTA's elements over its k-groups), the rest is summed
-    without loss, so |error| <= 512 * 2^-24 * sum |p_i p_j|."""
+    without loss, so |error| <= 512 * 2^-24 * sum |p_i p_j|.  An entry and its mirror image are the
+    same numbers added in 64 bits in another order: at most 608 of them."""
     rf = cuda_lib
     g = torch.Generator(device=DEV).manual_seed(F * 7 + E)
     buf = torch.randn(F * (E + pad) + shift, generator=g, device=DEV)
@@ -883,9 +884,22 @@ def test_frame_gram_tile_and_slice_edges(cuda_lib, F, E, pad, shift):
     rf.rf_frame_gram(P, G)
     torch.cuda.synchronize()
     p = P.double()
-    bound = 512 * 2.0 ** -24 * (p.abs() @ p.abs().t())
-    assert ((G - p @ p.t()).abs() <= bound).all()
-    assert torch.equal(G, G.t())
+    size = p.abs() @ p.abs().t()
+    assert ((G - p @ p.t()).abs() <= 512 * 2.0 ** -24 * size).all()
+    assert ((G - G.t()).abs() <= 2 * 608 * 2.0 ** -53 * size).all()
+
+
+@pytest.mark.parametrize("F,E", [(9, 1572863), (16, 1572865), (24, 2097153), (64, 786433)])
+def test_frame_gram_long_unaligned_rows(cuda_lib, F, E):
+    """Both sides of the rule for long rows off the 16-byte boundaries.  An fp32 chain has at most the
+    elements of one CTA of 304 or more, whole slices of 128, and one sum per k-group."""
+    rf = cuda_lib
+    P = torch.randn(F, E, generator=torch.Generator(device=DEV).manual_seed(E), device=DEV)
+    G = torch.empty(F, F, dtype=torch.float64, device=DEV)
+    rf.rf_frame_gram(P, G)
+    p = P.double()
+    chain = E / 304 + 128 + 32
+    assert ((G - p @ p.t()).abs() <= chain * 2.0 ** -24 * (p.abs() @ p.abs().t())).all()
 
 
 @pytest.mark.parametrize("F,E", [(9, 300), (33, 57600), (64, 3000), (64, 60000)])
