@@ -98,11 +98,13 @@ constexpr uint32_t kWaitLimitNs = 2000000000u;  // 2 s: no legitimate wait comes
 constexpr uint64_t kDrainLimitNs = 200000000ull;  // 0.2 s for in-flight copies at teardown
 constexpr float kRescaleLog2 = 8.0f;
 constexpr int kMaxSplit = 16;          // KV ranges per split item
-// KV tiles per range of a split item, at least: a merge costs about as much as the KV steps of
-// that many tiles (us per launch with at least 1, 2, 4, 8 tiles per range:
-// 4 x 64 tokens x 2 heads x 64 12.1, 8.8, 8.8, 8.8; 8 x 200 x 2 x 128 30.9, 26.3, 23.4, 23.7;
-// 5 x 400 x 3 x 64 18.6, 18.6, 17.4, 20.2; 21 x 200 x 3 x 128 37.4, 37.5, 30.8, 29.9).
-constexpr int kMinSplitTiles = 4;
+// KV tiles per piece where the tail is dealt out evenly, at least: a merge costs about as much as
+// the KV steps of that many tiles.  Equal ranges may be as short as one tile.  At least four tiles
+// there too are faster on short sequences (4 x 64 tokens x 2 heads x 64 8.1 us instead of 10.8,
+// 8 x 200 x 2 x 128 23.5 instead of 29.2), but further from the exact result: the largest
+// probability of every range is exactly 1 in bf16, so fewer ranges round more of the
+// probabilities (error of 48 drawn shapes 1.04 times as large, 1.09 at most).
+constexpr int kMinPiece = 4;
 constexpr int kMaxGrid = 1024;         // workspace is sized for at most this many CTAs
 // Block-masked launches: a ring of per-unit KV-tile bitmaps in shared memory, one bit per KV
 // tile (so at most kTLWords * 32 tiles of 128 keys), followed by the number of set bits.
@@ -189,13 +191,13 @@ struct Unit {
 constexpr int kSplitCost = 3, kEvenCost = 10;
 constexpr uint32_t kMinEvenShare = 12;  // KV tiles per CTA
 // KV tile, counted over the whole tail, where CTA k's share begins; no piece is shorter than
-// kMinSplitTiles.
+// kMinPiece.
 __device__ __forceinline__ uint32_t even_bound(const Sched& s, int nkv, int k) {
   // (fits 32 bits: the tail has fewer items than CTAs, and make_sched checks CTAs * nkv)
   const uint32_t v = k * s.even_q + k * s.even_r / gridDim.x;
   const uint32_t rem = v % static_cast<uint32_t>(nkv);
-  if (rem < kMinSplitTiles) return v - rem;
-  return nkv - rem < kMinSplitTiles ? v + (nkv - rem) : v;
+  if (rem < kMinPiece) return v - rem;
+  return nkv - rem < kMinPiece ? v + (nkv - rem) : v;
 }
 
 __device__ __forceinline__ Sched make_sched(const AttnParams& p) {
@@ -218,7 +220,7 @@ __device__ __forceinline__ Sched make_sched(const AttnParams& p) {
     const int tail = T - (rounds - 1) * G;
     int c = G / tail;
     if (c > kMaxSplit) c = kMaxSplit;
-    if (c > p.nkv / kMinSplitTiles) c = p.nkv / kMinSplitTiles;
+    if (c > p.nkv) c = p.nkv;
     const int busiest = c >= 2 ? (p.nkv + c - 1) / c + kSplitCost : p.nkv;
     if (p.ws_slots == 2 && 4 * tail > G && static_cast<uint32_t>(p.nkv) <= 0xFFFFFFFFu / G) {
       const uint32_t all = static_cast<uint32_t>(tail) * p.nkv, q = all / G;
@@ -879,8 +881,8 @@ __device__ __noinline__ int split_epilogue(const AttnParams& p, const Sched& sc,
   uint16_t* orow = p.O + token * p.o_row_stride + static_cast<int64_t>(u.h) * D;
   // A tile's partials are [D/4] float4 columns of 128 rows, then {m, l} of the rows: a warp's
   // stores and loads are 512 consecutive bytes.  (With each row's 528 bytes together and one
-  // range at a time in the merge, 4 x 256 tokens x 2 heads x 128 in 8 ranges took 69 us, now in 2
-  // ranges 17.6; 7 x 1003 x 2 x 128 in 7 ranges 69.6 -> 45.9.)
+  // range at a time in the merge, 4 x 256 tokens x 2 heads x 128 in 8 ranges took 69.0 us, now 22.9;
+  // 7 x 1003 x 2 x 128 in 2 ranges 69.7 -> 47.1.)
   float4* part = reinterpret_cast<float4*>(p.ws_part) +
                  static_cast<int64_t>(u.part * 2 + X) * (BM * C::kPartFloats / 4) + row;
 #pragma unroll 1
@@ -917,22 +919,17 @@ __device__ __noinline__ int split_epilogue(const AttnParams& p, const Sched& sc,
     };
     // O = sum_c 2^(m_c - M) O_c / sum_c 2^(m_c - M) l_c, M = max_c m_c (a split launch is
     // never block-masked: every m_c is finite)
-    // up to kMergeAhead loads per thread in flight: a merge is a chain of L2 round trips
-    constexpr int kMergeAhead = 4;
+    // all pieces' loads in flight: a merge is a chain of L2 round trips
+    float2 v[kMaxSplit];
+#pragma unroll
+    for (int c = 0; c < kMaxSplit; ++c)
+      v[c] = c < pieces.n ? ml(c) : make_float2(-INFINITY, 0.f);
     float M = -INFINITY, L = 0.f;
-    for (int c0 = 0; c0 < pieces.n; c0 += kMergeAhead) {
-      float2 v[kMergeAhead];
 #pragma unroll
-      for (int i = 0; i < kMergeAhead; ++i) v[i] = ml(min(c0 + i, pieces.n - 1));
-      float m_new = M;
+    for (int c = 0; c < kMaxSplit; ++c) M = fmaxf(M, v[c].x);
 #pragma unroll
-      for (int i = 0; i < kMergeAhead; ++i) m_new = fmaxf(m_new, v[i].x);
-      L *= ex2_approx(M - m_new);
-      M = m_new;
-#pragma unroll
-      for (int i = 0; i < kMergeAhead; ++i)
-        if (c0 + i < pieces.n) L += v[i].y * ex2_approx(v[i].x - M);
-    }
+    for (int c = 0; c < kMaxSplit; ++c)
+      if (c < pieces.n) L += v[c].y * ex2_approx(v[c].x - M);
     const float inv_L = 1.0f / L;
     float acc[32];
     auto add = [&](float wgt, const float4(&v)[8]) {
@@ -944,8 +941,9 @@ __device__ __noinline__ int split_epilogue(const AttnParams& p, const Sched& sc,
         acc[4 * q + 3] = fmaf(v[q].w, wgt, acc[4 * q + 3]);
       }
     };
-    // two blocks of 32 columns at a time, each with two ranges, or one block with
-    // kMergeAhead ranges at a time
+    // up to kMergeAhead columns' loads in flight: two blocks of 32 columns at a time, each with two
+    // ranges, or one block with kMergeAhead ranges at a time
+    constexpr int kMergeAhead = 4;
     const int blocks = pieces.n <= 2 ? 2 : 1, at_once = kMergeAhead / blocks;
 #pragma unroll 1
     for (int cc = 0; cc < D / 32; cc += blocks) {

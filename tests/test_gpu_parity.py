@@ -667,6 +667,36 @@ def test_attn_dealt_evenly(cuda_lib, F, N, H, d, A):
     assert all((outs[0].float() - o.float()).abs().max().item() < 1e-2 for o in outs[2:])
 
 
+@pytest.mark.parametrize("F,N,H,d", [
+    (4, 64, 2, 64),     # two ranges
+    (3, 300, 2, 64),    # eight ranges, the last key tile of four keys
+    (8, 256, 1, 128),   # sixteen ranges
+])
+def test_attn_short_split_rounds_each_tile_by_its_own_max(cuda_lib, F, N, H, d):
+    """A short sequence on an idle chip is split down to ranges of one key tile, and the probabilities
+    of a range are rounded to bf16 relative to the range's own max.  Against that, evaluated in
+    64 bits, only the output's rounding is left: 2^-9 of a value at most, and less than 2^-9
+    in the 2-norm even with the few probabilities that the hardware exponential rounds the other
+    way.  Ranges of any other length round about all of them differently."""
+    rf = cuda_lib
+    Q, K, V = _qkv(F * N, H, d, seed=F * 7 + N)
+    mask = [1] + [0] * (F - 1)
+    scale = 1.0 / math.sqrt(d)
+    O, _ = _run_attn(rf, Q, K, V, F, N, mask, scale, split=True)
+    x = torch.einsum("qhd,khd->hqk", Q[:N].double(), K.double()) * (scale * math.log2(math.e))
+    top, acc, total = x.amax(-1, keepdim=True), 0.0, 0.0
+    for k0 in range(0, F * N, 128):
+        t = x[:, :, k0:k0 + 128]
+        m = t.amax(-1, keepdim=True)
+        p = torch.exp2(t - m)
+        acc = acc + torch.exp2(m - top) * torch.einsum(
+            "hqk,khd->hqd", p.to(torch.bfloat16).double(), V[k0:k0 + 128].double())
+        total = total + torch.exp2(m - top) * p.sum(-1, keepdim=True)
+    want = (acc / total).permute(1, 0, 2)
+    err = ((O[:N].double() - want).norm() / want.norm()).item()
+    assert err < 2.0 ** -9, err
+
+
 def _pipeline_against_device_path(F, N, H, d, E, plan_args, Q, K0, V0, vel, z0, scale, nsteps,
                                   depth):
     """The same steps on device-resident inputs (StepCore, fresh K/V rows written before each
