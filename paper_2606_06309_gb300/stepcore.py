@@ -133,19 +133,22 @@ class StepCore:
         frames' rows of K and V are overwritten with their projection before the attention.
 
         One call and two launches: all but the attention in the first.  4 x 64 tokens, 2 heads:
-        23.4 us per step (host and launches) against 33.4 as five calls."""
-        stream = _stream(stream)  # looked up once
-        p = self.plan
-        try:
-            rf_step_core(_row(p.mask, s), _row(p.cur_slot, s), _row(p.alpha, s), _row(p.beta, s),
-                         _row(p.dt, s), self.F, self.N, self.E, self.H, self.d, self.active,
-                         self.skipped, self.token_idx, self.counts, self.ctx, self.z2, v, self.Kc,
-                         self.Vc, O, lse, Q, K, V, Q.stride(0),
-                         0 if self.Kc is None else K.stride(0), O.stride(0), scale,
-                         self.workspace, self.status, stream)
-            return
-        except RFError:
-            pass  # call by call, so that the error is the one of the call at fault
+        23.4 us per step (host and launches) against 33.4 as five calls.  Where compact, project,
+        project_kv, attn or step has been replaced, in a subclass or on the object, the five are
+        called instead."""
+        if self._own_parts():
+            at = _stream(stream)  # looked up once
+            p = self.plan
+            try:
+                rf_step_core(_row(p.mask, s), _row(p.cur_slot, s), _row(p.alpha, s),
+                             _row(p.beta, s), _row(p.dt, s), self.F, self.N, self.E, self.H,
+                             self.d, self.active, self.skipped, self.token_idx, self.counts,
+                             self.ctx, self.z2, v, self.Kc, self.Vc, O, lse, Q, K, V, Q.stride(0),
+                             0 if self.Kc is None else K.stride(0), O.stride(0), scale,
+                             self.workspace, self.status, at)
+                return
+            except RFError:
+                pass  # call by call, so that the error is the one of the call at fault
         self.compact(s, stream)
         self.project(s, stream)
         if self.Kc is not None:
@@ -153,10 +156,18 @@ class StepCore:
         self.attn(O, Q, K, V, scale, lse, stream)
         self.step(s, v, stream)
 
+    def _own_parts(self) -> bool:
+        """Whether the parts of a step are this class's own methods."""
+        cls = type(self)
+        return ((cls.compact, cls.project, cls.project_kv, cls.attn, cls.step) == _PARTS
+                and self.__dict__.keys().isdisjoint(_PART_NAMES))
+
     @property
     def launches_per_step(self) -> int:
-        """Of run() (the parts called one by one are five, or four without the cache)."""
-        return 2
+        """Of run(): two.  Where one of the parts has been replaced, or where buffers of the caller's
+        overlap in a way that needs the parts' order (which is not seen here), each part is a
+        launch: five, or four without the cache."""
+        return 2 if self._own_parts() else 5 if self.Kc is not None else 4
 
     def capture_trajectory(self, vels, O, Q, K, V, scale: float, steps=None):
         """Record steps 0..S-1 (all launches of each) into one CUDA graph and return it.
@@ -174,6 +185,10 @@ class StepCore:
             for s in range(S):
                 self.run(s, vels[s], O, Q, K, V, scale)
         return g
+
+
+_PART_NAMES = ("compact", "project", "project_kv", "attn", "step")
+_PARTS = tuple(getattr(StepCore, name) for name in _PART_NAMES)
 
 
 class HostPipeline:

@@ -262,3 +262,64 @@ def test_plan_row_addresses():
         for s in (7, -8):
             with pytest.raises(IndexError):
                 _row(t, s)
+
+
+def _host_step_core(cls, **kw):
+    """A step core of host tensors, for tests that replace every call of the library."""
+    from paper_2606_06309_gb300.stepcore import upload_plan
+    plan = upload_plan(3, 2, [1, 0, 1], [1, 1], 0, "cpu")
+    return cls(3, 4, 8, 1, 64, plan, "cpu", split_kv=False, **kw)
+
+
+@pytest.mark.parametrize("part", ["compact", "project", "project_kv", "attn", "step"])
+@pytest.mark.parametrize("how", ["subclass", "object", "class"])
+def test_run_calls_replaced_parts(rf, monkeypatch, part, how):
+    """StepCore.run takes the fused call only where all five parts are its own: a part replaced in a
+    subclass, on the object or on the class itself is called, with run's own arguments."""
+    import torch
+
+    from paper_2606_06309_gb300 import stepcore
+    calls = []
+    for name in ("rf_schedule_compact", "rf_project", "rf_project_kv", "rf_attn", "rf_step",
+                 "rf_step_core"):
+        monkeypatch.setattr(stepcore, name, lambda *a, name=name, **k: calls.append(name))
+    inner = getattr(stepcore.StepCore, part)
+
+    def outer(self, *a, **k):
+        calls.append((part, a[-1]))
+        return inner(self, *a, **k)
+
+    cls = stepcore.StepCore
+    if how == "subclass":
+        cls = type("Sub", (cls,), {part: outer})
+    elif how == "class":
+        monkeypatch.setattr(cls, part, outer)
+    core = _host_step_core(cls)
+    if how == "object":
+        setattr(core, part, outer.__get__(core))
+    x = torch.zeros(12, 1, 64, dtype=torch.bfloat16)
+
+    class Stream:
+        cuda_stream = 0
+
+    stream = Stream()
+    core.run(0, torch.zeros(3, 8), x, x, x, x, 0.1, stream=stream)
+    want = ["rf_schedule_compact", "rf_project", "rf_project_kv", "rf_attn", "rf_step"]
+    at = ["compact", "project", "project_kv", "attn", "step"].index(part)
+    want.insert(at, (part, stream))
+    assert calls == want
+    assert core.launches_per_step == 5
+
+
+def test_run_of_the_class_itself_is_one_call(rf, monkeypatch):
+    import torch
+
+    from paper_2606_06309_gb300 import stepcore
+    calls = []
+    monkeypatch.setattr(stepcore, "rf_step_core", lambda *a: calls.append(a))
+    x = torch.zeros(12, 1, 64, dtype=torch.bfloat16)
+    for cls in (stepcore.StepCore, type("Sub", (stepcore.StepCore,), {"more": lambda self: 1})):
+        core = _host_step_core(cls)
+        core.run(1, torch.zeros(3, 8), x, x, x, x, 0.1, stream=7)
+        assert core.launches_per_step == 2
+    assert len(calls) == 2 and all(a[-1] == 7 for a in calls)
