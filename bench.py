@@ -41,12 +41,12 @@ FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustain
 # dram__bytes_write.sum), per workload.  A figure is reported only while the kernel source
 # still has the hash it was measured with.
 ATTN_TRAFFIC = {
-    "small": {"bytes_per_launch": 189169536, "code_sha256_rf_attn_cu":
-              "92a1dbec07495fedbf7ec1a533a1c423e3e63add2b39703739909819e94c3610",
+    "small": {"bytes_per_launch": 189199821, "code_sha256_rf_attn_cu":
+              "e29cddfceda150ccd907e3adee9662e3e173fa0b2c6362293ebd84716bdf8ba3",
               "launch": "average over the 20 launches of one trajectory of the small workload "
                         "(10 with all 13 frames active, 10 with the 4 keyframes)"},
-    "long": {"bytes_per_launch": 4743453773, "code_sha256_rf_attn_cu":
-             "92a1dbec07495fedbf7ec1a533a1c423e3e63add2b39703739909819e94c3610",
+    "long": {"bytes_per_launch": 4397522801, "code_sha256_rf_attn_cu":
+             "e29cddfceda150ccd907e3adee9662e3e173fa0b2c6362293ebd84716bdf8ba3",
              "launch": "average over the 50 launches of one trajectory of the long workload "
                        "(21 with all 33 frames active, 29 with the 6 keyframes)"},
 }

@@ -295,8 +295,11 @@ rf_status rf_step(float* d_z2, const uint8_t* d_cur_slot, const float* d_v, cons
  * are given; both NULL: without the cache), rf_attn and rf_step, with the arguments of those
  * calls and D = H*d.  Every argument is checked before anything is enqueued; the first error, in
  * that order, is returned.  Same results as the five calls, in two launches: everything but the
- * attention shares one.  Where the buffers overlap in a way that needs the calls' order (d_v a
- * view of d_ctx or of d_O, say), each part is launched by itself in that order.
+ * attention shares one.  The Euler update then goes in front of the attention, so whatever of the
+ * attention can be refused (the tensor maps included) is refused before the first launch, and
+ * only a failed launch of the attention itself leaves the rest of the step done.
+ * Where the buffers overlap in a way that needs the calls' order (d_v a view of d_ctx or of d_O,
+ * say), each part is launched by itself in that order.
  *   qkv_row_stride  of d_Q, d_K, d_V in the attention; kv_row_stride of d_K, d_V in the cache step
  */
 rf_status rf_step_core(const uint8_t* d_mask, const uint8_t* d_cur_slot, const float* d_alpha,

@@ -1486,11 +1486,12 @@ int64_t workspace_bytes(int d, int grid, int slots) {
 }
 
 template <int D, bool MASKED>
-rf_status launch(const CUtensorMap& q, const CUtensorMap& q128, const CUtensorMap& k,
-                 const CUtensorMap& v,
-                 const AttnParams& p, int grid, const DeviceInfo& di, cudaStream_t stream) {
-  using C = Cfg<D>;
-  constexpr int smem = MASKED ? C::kSmemBytesMasked : C::kSmemBytes;
+constexpr int kSmem = MASKED ? Cfg<D>::kSmemBytesMasked : Cfg<D>::kSmemBytes;
+
+// What the kernel needs once per device, before its first launch.
+template <int D, bool MASKED>
+rf_status prepare(const DeviceInfo& di) {
+  constexpr int smem = kSmem<D, MASKED>;
   static bool attr_set[64] = {};
   if (smem > di.max_smem_optin) return fail(RF_ERR_UNSUPPORTED, "shared memory");
   if (!attr_set[di.device]) {
@@ -1499,7 +1500,13 @@ rf_status launch(const CUtensorMap& q, const CUtensorMap& q128, const CUtensorMa
       return fail(RF_ERR_CUDA, "cudaFuncSetAttribute(attn_kernel)", e);
     attr_set[di.device] = true;
   }
-  attn_kernel<D, MASKED><<<grid, kThreads, smem, stream>>>(q, q128, k, v, p);
+  return RF_OK;
+}
+
+template <int D, bool MASKED>
+rf_status launch(const CUtensorMap& q, const CUtensorMap& q128, const CUtensorMap& k,
+                 const CUtensorMap& v, const AttnParams& p, int grid, cudaStream_t stream) {
+  attn_kernel<D, MASKED><<<grid, kThreads, kSmem<D, MASKED>, stream>>>(q, q128, k, v, p);
   return launch_status("attn_kernel launch");
 }
 
@@ -1558,11 +1565,12 @@ rf_status check_attn_args(const void* d_O, const void* d_Q, const void* d_K, con
   return RF_OK;
 }
 
+// Nothing is enqueued before the last thing that can be refused; `front` is enqueued first.
 rf_status attn_impl(void* d_O, float* d_lse, const void* d_Q, const void* d_K, const void* d_V,
                     int64_t qkv_row_stride, int64_t o_row_stride, int F, int N, int H, int d,
                     const int32_t* d_active, const int32_t* d_counts, float softmax_scale,
                     const uint8_t* d_block_mask, void* d_workspace, int64_t workspace_bytes_given,
-                    int32_t* d_status, rf_stream_t stream) {
+                    int32_t* d_status, rf_stream_t stream, const Front* front = nullptr) {
   DeviceInfo di;
   if (rf_status st = check_attn_args(d_O, d_Q, d_K, d_V, qkv_row_stride, o_row_stride, F, N, H,
                                      d, d_active, d_counts, softmax_scale, d_block_mask,
@@ -1571,6 +1579,9 @@ rf_status attn_impl(void* d_O, float* d_lse, const void* d_Q, const void* d_K, c
   const int64_t S_tok = static_cast<int64_t>(F) * N;
   const int64_t Np = (static_cast<int64_t>(N) + 7) / 8 * 8;
 
+  if (rf_status st = d_block_mask ? (d == 128 ? prepare<128, true>(di) : prepare<64, true>(di))
+                                  : (d == 128 ? prepare<128, false>(di) : prepare<64, false>(di)))
+    return st;
   CUtensorMap mq, mq128, mk, mv;
   if (rf_status st = make_map(&mq, d_Q, d, H, static_cast<int>(S_tok), qkv_row_stride, 8)) return st;
   if (rf_status st = make_map(&mq128, d_Q, d, H, static_cast<int>(S_tok), qkv_row_stride, BM))
@@ -1612,6 +1623,8 @@ rf_status attn_impl(void* d_O, float* d_lse, const void* d_Q, const void* d_K, c
   p.nkv = static_cast<int>((S_tok + BN - 1) / BN);
   p.scale_log2 = static_cast<float>(static_cast<double>(softmax_scale) * 1.4426950408889634);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  if (front)
+    if (rf_status st = front->launch(front->arg, s)) return st;
   if (d_block_mask) {
     // With a workspace: costs and the longest-first order of the items in its partial-row
     // area (unused by block-masked launches, which never split), when it holds them.
@@ -1635,11 +1648,11 @@ rf_status attn_impl(void* d_O, float* d_lse, const void* d_Q, const void* d_K, c
       if (rf_status st = launch_status("lpt_prepass_kernel launch")) return st;
       p.lpt_order = order;
     }
-    return d == 128 ? launch<128, true>(mq, mq128, mk, mv, p, grid, di, s)
-                    : launch<64, true>(mq, mq128, mk, mv, p, grid, di, s);
+    return d == 128 ? launch<128, true>(mq, mq128, mk, mv, p, grid, s)
+                    : launch<64, true>(mq, mq128, mk, mv, p, grid, s);
   }
-  return d == 128 ? launch<128, false>(mq, mq128, mk, mv, p, grid, di, s)
-                  : launch<64, false>(mq, mq128, mk, mv, p, grid, di, s);
+  return d == 128 ? launch<128, false>(mq, mq128, mk, mv, p, grid, s)
+                  : launch<64, false>(mq, mq128, mk, mv, p, grid, s);
 }
 }  // namespace
 
@@ -1652,6 +1665,17 @@ rf_status rf::attn_check(const void* d_O, const void* d_Q, const void* d_K, cons
   return check_attn_args(d_O, d_Q, d_K, d_V, qkv_row_stride, o_row_stride, F, N, H, d, d_active,
                          d_counts, softmax_scale, nullptr, d_workspace, workspace_bytes_given,
                          &di);
+}
+
+rf_status rf::attn_behind(const Front& front, void* d_O, float* d_lse, const void* d_Q,
+                          const void* d_K, const void* d_V, int64_t qkv_row_stride,
+                          int64_t o_row_stride, int F, int N, int H, int d,
+                          const int32_t* d_active, const int32_t* d_counts, float softmax_scale,
+                          void* d_workspace, int64_t workspace_bytes_given, int32_t* d_status,
+                          rf_stream_t stream) {
+  return attn_impl(d_O, d_lse, d_Q, d_K, d_V, qkv_row_stride, o_row_stride, F, N, H, d, d_active,
+                   d_counts, softmax_scale, nullptr, d_workspace, workspace_bytes_given, d_status,
+                   stream, &front);
 }
 
 extern "C" rf_status rf_attn(void* d_O, float* d_lse, const void* d_Q, const void* d_K,

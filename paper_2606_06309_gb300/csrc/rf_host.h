@@ -36,4 +36,18 @@ rf_status attn_check(const void* d_O, const void* d_Q, const void* d_K, const vo
                      const int32_t* d_active, const int32_t* d_counts, float softmax_scale,
                      const void* d_workspace, int64_t workspace_bytes);
 
+// Work that goes in front of an attention on its stream.
+struct Front {
+  rf_status (*launch)(const void* arg, cudaStream_t stream);
+  const void* arg;
+};
+
+// rf_attn behind `front`, which is launched once nothing is left that could be refused: arguments
+// checked, tensor maps made, kernel attributes set.
+rf_status attn_behind(const Front& front, void* d_O, float* d_lse, const void* d_Q,
+                      const void* d_K, const void* d_V, int64_t qkv_row_stride,
+                      int64_t o_row_stride, int F, int N, int H, int d, const int32_t* d_active,
+                      const int32_t* d_counts, float softmax_scale, void* d_workspace,
+                      int64_t workspace_bytes, int32_t* d_status, rf_stream_t stream);
+
 }  // namespace rf

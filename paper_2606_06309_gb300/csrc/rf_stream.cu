@@ -478,6 +478,14 @@ __global__ void __launch_bounds__(kKvThreads) front_kernel(const __grid_constant
            p.F, p.N, p.D, f, p.mask[f] != 0, base);
 }
 
+rf_status launch_front(const void* arg, cudaStream_t stream) {
+  // an error that an earlier call left behind is reported while nothing has been enqueued
+  if (rf_status st = launch_status("before rf_step_core")) return st;
+  const FrontParams& p = *static_cast<const FrontParams*>(arg);
+  front_kernel<<<1 + p.n_tok + p.n_lat + 2 * p.n_kv, kKvThreads, 0, stream>>>(p);
+  return launch_status("front_kernel launch");
+}
+
 // Address ranges of a step's buffers, to see whether its parts may share a launch.
 enum : uint32_t {
   kReads = 1,        // read by front_kernel
@@ -737,24 +745,22 @@ extern "C" rf_status rf_step_core(
     p.n_tok = static_cast<uint32_t>(tok * F);
     p.n_lat = static_cast<uint32_t>(lat * F);
     p.n_kv = static_cast<uint32_t>(kv * F);
-    front_kernel<<<1 + p.n_tok + p.n_lat + 2 * p.n_kv, kKvThreads, 0,
-                   reinterpret_cast<cudaStream_t>(stream)>>>(p);
-    if (rf_status st = launch_status("front_kernel launch")) return st;
-  } else {
-    if (rf_status st = rf_schedule_compact(d_mask, F, N, d_active, d_skipped, d_token_idx,
-                                           d_counts, stream))
-      return st;
-    if (rf_status st = rf_project(d_ctx, d_z2, d_cur_slot, d_alpha, d_beta, F, E, stream))
-      return st;
-    if (cache)
-      if (rf_status st = rf_project_kv(d_K, d_V, kv_row_stride, d_Kc, d_Vc, d_cur_slot, d_alpha,
-                                       d_beta, d_active, d_skipped, d_counts, F, N, D, stream))
-        return st;
+    // the Euler update goes in front of the attention, so that must be able to follow
+    return attn_behind(Front{launch_front, &p}, d_O, d_lse, d_Q, d_K, d_V, qkv_row_stride,
+                       o_row_stride, F, N, H, d, d_active, d_counts, softmax_scale, d_workspace,
+                       workspace_bytes, d_status, stream);
   }
+  if (rf_status st = rf_schedule_compact(d_mask, F, N, d_active, d_skipped, d_token_idx, d_counts,
+                                         stream))
+    return st;
+  if (rf_status st = rf_project(d_ctx, d_z2, d_cur_slot, d_alpha, d_beta, F, E, stream)) return st;
+  if (cache)
+    if (rf_status st = rf_project_kv(d_K, d_V, kv_row_stride, d_Kc, d_Vc, d_cur_slot, d_alpha,
+                                     d_beta, d_active, d_skipped, d_counts, F, N, D, stream))
+      return st;
   if (rf_status st = rf_attn(d_O, d_lse, d_Q, d_K, d_V, qkv_row_stride, o_row_stride, F, N, H, d,
                              d_active, d_counts, softmax_scale, d_workspace, workspace_bytes,
                              d_status, stream))
     return st;
-  return together ? RF_OK
-                  : rf_step(d_z2, d_cur_slot, d_v, d_dt, d_active, d_counts, F, E, stream);
+  return rf_step(d_z2, d_cur_slot, d_v, d_dt, d_active, d_counts, F, E, stream);
 }

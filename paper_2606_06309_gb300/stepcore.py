@@ -30,6 +30,9 @@ from . import (RFError, _stream, rf_attn, rf_attn_workspace_bytes, rf_pipeline_b
                rf_project_kv, rf_schedule_compact, rf_step, rf_step_core)
 
 
+_RF_ERR_CUDA = 4  # a CUDA call or a launch failed
+
+
 @dataclass
 class Plan:
     mask: torch.Tensor      # [S, F] uint8
@@ -147,8 +150,11 @@ class StepCore:
                              0 if self.Kc is None else K.stride(0), O.stride(0), scale,
                              self.workspace, self.status, at)
                 return
-            except RFError:
-                pass  # call by call, so that the error is the one of the call at fault
+            except RFError as e:
+                if e.status == _RF_ERR_CUDA:  # not of an argument: some of it may have been enqueued
+                    raise
+            # refused, with nothing enqueued: call by call, so that the error is the one of the
+            # call at fault
         self.compact(s, stream)
         self.project(s, stream)
         if self.Kc is not None:

@@ -323,3 +323,29 @@ def test_run_of_the_class_itself_is_one_call(rf, monkeypatch):
         core.run(1, torch.zeros(3, 8), x, x, x, x, 0.1, stream=7)
         assert core.launches_per_step == 2
     assert len(calls) == 2 and all(a[-1] == 7 for a in calls)
+
+
+@pytest.mark.parametrize("status", [1, 2, 3, 4])
+def test_run_repeats_a_refused_step_only(rf, monkeypatch, status):
+    """An argument that the fused call refuses is left to the call at fault; a failed CUDA call, after
+    which some of the step may have been enqueued, is raised with nothing repeated."""
+    import torch
+
+    from paper_2606_06309_gb300 import stepcore
+    calls = []
+    for name in ("rf_schedule_compact", "rf_project", "rf_project_kv", "rf_attn", "rf_step"):
+        monkeypatch.setattr(stepcore, name, lambda *a, name=name: calls.append(name))
+
+    def fused(*a):
+        raise rf.RFError("rf_step_core", status)
+
+    monkeypatch.setattr(stepcore, "rf_step_core", fused)
+    core = _host_step_core(stepcore.StepCore)
+    x = torch.zeros(12, 1, 64, dtype=torch.bfloat16)
+    if status == 4:
+        with pytest.raises(rf.RFError, match="rf_step_core failed"):
+            core.run(0, torch.zeros(3, 8), x, x, x, x, 0.1, stream=0)
+        assert calls == []
+    else:
+        core.run(0, torch.zeros(3, 8), x, x, x, x, 0.1, stream=0)
+        assert calls == ["rf_schedule_compact", "rf_project", "rf_project_kv", "rf_attn", "rf_step"]

@@ -1087,6 +1087,24 @@ def test_step_core_errors_are_those_of_the_call_at_fault(cuda_lib):
     assert torch.equal(core.z2, torch.ones_like(core.z2))
 
 
+def test_step_core_refused_tensor_map_leaves_the_state(cuda_lib):
+    """A row stride of 2^40 bytes, which only the encoding of the tensor maps refuses: the step raises
+    and nothing of it has been done, the Euler update in front of the attention above all."""
+    from paper_2606_06309_gb300.stepcore import StepCore, upload_plan
+    core = StepCore(1, 1, 4, 1, 64, upload_plan(1, 2, [1], [1, 1], 0, DEV), DEV)
+    core.set_state(torch.ones(1, 4, device=DEV))
+    x = torch.ones(1, 1, 64, dtype=torch.bfloat16, device=DEV)
+    far = x.as_strided((1, 1, 64), (2 ** 39, 64, 1))  # one row: the stride reaches no memory
+    v = torch.ones(1, 4, device=DEV)
+    kept = [t.clone() for t in (core.z2, core.Kc, core.Vc, core.ctx, core.counts)]
+    with pytest.raises(cuda_lib.RFError, match="cuTensorMapEncodeTiled"):
+        core.run(0, v, x.clone(), far, x.clone(), x.clone(), 0.1)
+    for a, b in zip((core.z2, core.Kc, core.Vc, core.ctx, core.counts), kept):
+        assert torch.equal(a, b)
+    core.run(0, v, x.clone(), x, x.clone(), x.clone(), 0.1)
+    assert not torch.equal(core.z2, kept[0])
+
+
 # ---------------------------------------------------------------------------
 # rf_attn_block_masked: frame mask x token block mask (Appendix D)
 # ---------------------------------------------------------------------------
