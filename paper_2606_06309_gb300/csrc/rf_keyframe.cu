@@ -15,8 +15,10 @@
 // threads read neighbouring rows, and KG = 2^n k-groups of tiles fill up to 256 threads, each
 // group taking every KG-th quad of elements.  At the end the k-groups are summed in shared
 // memory, then the two CTAs of a cluster through distributed shared memory, both as
-// unevaluated pairs of floats (the fp64 units are few), and one fp64 atomic per entry and
-// cluster reaches the result.
+// unevaluated pairs of floats (the fp64 units are few; a sum past their range is made again in
+// 64 bits), and one fp64 atomic per entry and cluster reaches the result.  So only a thread's own
+// chain of multiply-adds has the range of fp32: at most 96 of the 384 elements of a short
+// CTA (four k-groups, above 56 frames), or a quarter of a long one's.
 //
 // What bounds it: at latent width (33 x 57600) launches, the final sums and the atomics; at
 // hidden width instruction issue and shared-memory reads.  A tile of T x T costs 2T 16-byte
@@ -207,9 +209,16 @@ __global__ void __launch_bounds__(kGramThreads, 2)
     const int a = (e / T) % T, b = e % T;
     const int fi = ti + a * groups, fj = tj + b * groups;
     if (fi < F && fj < F && (ti != tj || a <= b)) {
-      // an infinite or undefined sum is in hi; the rounding errors beside it are not numbers
-      const double t = isfinite(hi) ? static_cast<double>(hi) + static_cast<double>(lo)
-                                    : static_cast<double>(hi);
+      double t = static_cast<double>(hi) + static_cast<double>(lo);
+      if (!isfinite(t)) {
+        // a pair of floats has the range of one: add the k-groups' sums again in 64 bits, which
+        // leaves infinite and undefined only what is infinite or undefined in one k-group
+        t = 0.0;
+        for (int c = 0; c < kGramCluster; ++c) {
+          const float* sums = cluster.map_shared_rank(part + e, c);
+          for (int q = 0; q < kgroups; ++q) t += static_cast<double>(sums[q * entries]);
+        }
+      }
       atomicAdd(out + static_cast<int64_t>(fi) * F + fj, t);
       if (fi != fj) atomicAdd(out + static_cast<int64_t>(fj) * F + fi, t);
     }

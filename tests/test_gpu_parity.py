@@ -949,6 +949,24 @@ def test_frame_gram_infinities_and_nan(cuda_lib, F, E):
     assert torch.equal(G[want.isinf()], want[want.isinf()])
 
 
+@pytest.mark.parametrize("F,E", [(1, 57600), (9, 24960), (33, 57600), (41, 57600), (64, 57600)])
+def test_frame_gram_sums_past_the_range_of_fp32(cuda_lib, F, E):
+    """Proxies of 1.5e18: 128 products of them (an fp32 sum of the plain CTAs' kernel) stay below the
+    largest float, 3.4e38, and what a CTA of 384 elements or more sums does not.  Alternating
+    signs in one frame: sums that come back into the range.  Relative error as of any fp32 chain
+    of at most 128 elements."""
+    rf = cuda_lib
+    P = torch.full((F, E), 1.5e18, device=DEV)
+    P[F // 2, 1::2] *= -1.0
+    P *= 0.5 + 0.5 * torch.rand(F, E, generator=torch.Generator(device=DEV).manual_seed(F),
+                                device=DEV)
+    G = torch.empty(F, F, dtype=torch.float64, device=DEV)
+    rf.rf_frame_gram(P, G)
+    p = P.double()
+    assert torch.isfinite(G).all()
+    assert ((G - p @ p.t()).abs() <= 128 * 2.0 ** -24 * (p.abs() @ p.abs().t())).all()
+
+
 def test_keyframes_from_device_gram_match_oracle(cuda_lib):
     """Scene-structured proxies (5 scenes over 21 frames of 3600 tokens x 16 channels):
     the keyframes are the scene starts, as the oracle's Algorithm 1 finds them."""
