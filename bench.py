@@ -41,12 +41,12 @@ FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustain
 # dram__bytes_write.sum), per workload.  A figure is reported only while the kernel source
 # still has the hash it was measured with.
 ATTN_TRAFFIC = {
-    "small": {"bytes_per_launch": 189199821, "code_sha256_rf_attn_cu":
-              "e29cddfceda150ccd907e3adee9662e3e173fa0b2c6362293ebd84716bdf8ba3",
+    "small": {"bytes_per_launch": 189168358, "code_sha256_rf_attn_cu":
+              "01318bd55075869180967589f10aa7c55463b5b85f7b8d6f0de3821f55d0cf34",
               "launch": "average over the 20 launches of one trajectory of the small workload "
                         "(10 with all 13 frames active, 10 with the 4 keyframes)"},
-    "long": {"bytes_per_launch": 4397522801, "code_sha256_rf_attn_cu":
-             "e29cddfceda150ccd907e3adee9662e3e173fa0b2c6362293ebd84716bdf8ba3",
+    "long": {"bytes_per_launch": 5022970542, "code_sha256_rf_attn_cu":
+             "01318bd55075869180967589f10aa7c55463b5b85f7b8d6f0de3821f55d0cf34",
              "launch": "average over the 50 launches of one trajectory of the long workload "
                        "(21 with all 33 frames active, 29 with the 6 keyframes)"},
 }
@@ -66,12 +66,14 @@ def _peaks():
 
 
 def _code_sha(path):
-    """sha256 of a C++/CUDA source with its // comments and blank lines removed: counters
-    recorded for a kernel stay attached to it while only comments change.  (The source holds
-    no "//" inside string literals.)"""
+    """sha256 of a C++/CUDA source and the .cuh files it includes, with // comments and blank lines
+    removed: counters recorded for a kernel stay attached to it while only comments change.
+    (The sources hold no "//" inside string literals.)"""
     lines = []
     for line in open(path, encoding="utf-8"):
         code = line.split("//", 1)[0].rstrip()
+        if code.startswith('#include "') and code.endswith('.cuh"'):
+            code += " " + _code_sha(os.path.join(os.path.dirname(path), code.split('"')[1]))
         if code:
             lines.append(code)
     return hashlib.sha256("\n".join(lines).encode()).hexdigest()

@@ -203,6 +203,24 @@ def test_header_is_a_c_abi(rf, tmp_path):
     assert r.returncode == 0 and r.stdout.startswith("ok"), (r.returncode, r.stdout, r.stderr)
 
 
+def test_attention_schedules(tmp_path):
+    """The schedule arithmetic of the attention kernel over 14,000 random launches on grids of 1 to
+    1024 CTAs (tests/c_abi/sched_check.cpp says what is checked)."""
+    import shutil
+    import subprocess
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("no C++ compiler")
+    exe = tmp_path / "sched_check"
+    cmd = [gxx, "-O2", "-std=c++17", "-Wall", "-Wextra", "-Werror", "-I",
+           os.path.join(ROOT, "paper_2606_06309_gb300", "csrc"),
+           os.path.join(ROOT, "tests", "c_abi", "sched_check.cpp"), "-o", str(exe)]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0 and r.stdout.startswith("ok"), (r.returncode, r.stdout, r.stderr)
+
+
 def _scene_proxies(F=21, E=960, starts=(0, 4, 9, 13, 17), noise=0.3, seed=0):
     rng = np.random.default_rng(seed)
     base = rng.standard_normal((len(starts), E))
