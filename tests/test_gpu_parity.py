@@ -896,6 +896,21 @@ def test_frame_gram_matches_fp64_matmul(cuda_lib, F, E, ld):
     assert err.max() < 1e-5, err.max()
 
 
+def _gram_of_integers(rf, F, E, pad, shift, seed):
+    """The Gram matrix of whole numbers 1 to 3 of either sign equals the 64-bit one exactly: every fp32
+    sum is a whole number of at most 9 per element, and no CTA has 2^24 / 9 elements.  Each element
+    is at least 1 of its diagonal entry, so one left out or taken twice anywhere shows."""
+    g = torch.Generator(device=DEV).manual_seed(seed)
+    buf = torch.randint(1, 4, (F * (E + pad) + shift,), generator=g, device=DEV).float()
+    buf *= torch.randint(0, 2, buf.shape, generator=g, device=DEV) * 2.0 - 1.0
+    P = buf[shift:].view(F, E + pad)[:, :E]
+    G = torch.full((F, F), 9.0, dtype=torch.float64, device=DEV)
+    rf.rf_frame_gram(P, G)
+    p = P.double()
+    want = p @ p.t()
+    assert torch.equal(G, want), (G - want).abs().max().item()
+
+
 @pytest.mark.parametrize("F", [1, 8, 9, 16, 17, 40, 41, 48, 64])
 @pytest.mark.parametrize("E,pad,shift", [(1, 0, 0), (127, 1, 0), (129, 3, 1), (3071, 1, 0),
                                          (20479, 1, 0), (20480, 0, 0), (24575, 1, 0),
@@ -905,7 +920,8 @@ def test_frame_gram_tile_and_slice_edges(cuda_lib, F, E, pad, shift):
     """Frame groups of 8, slices cut short, rows and bases off the 16-byte boundaries.  Each fp32
     chain has at most 512 products (a CTA's elements over its k-groups), the rest is summed
     without loss, so |error| <= 512 * 2^-24 * sum |p_i p_j|.  An entry and its mirror image are the
-    same numbers added in 64 bits in another order: at most 608 of them."""
+    same numbers added in 64 bits in another order: at most 608 of them.  That bound is no
+    smaller than an element of a long row; whole numbers show that none is lost or doubled."""
     rf = cuda_lib
     g = torch.Generator(device=DEV).manual_seed(F * 7 + E)
     buf = torch.randn(F * (E + pad) + shift, generator=g, device=DEV)
@@ -917,12 +933,14 @@ def test_frame_gram_tile_and_slice_edges(cuda_lib, F, E, pad, shift):
     size = p.abs() @ p.abs().t()
     assert ((G - p @ p.t()).abs() <= 512 * 2.0 ** -24 * size).all()
     assert ((G - G.t()).abs() <= 2 * 608 * 2.0 ** -53 * size).all()
+    _gram_of_integers(rf, F, E, pad, shift, E)
 
 
 @pytest.mark.parametrize("F,E", [(9, 1572863), (16, 1572865), (24, 2097153), (64, 786433)])
 def test_frame_gram_long_unaligned_rows(cuda_lib, F, E):
     """Both sides of the rule for long rows off the 16-byte boundaries.  An fp32 chain has at most the
-    elements of one CTA of 304 or more, whole slices of 128, and one sum per k-group."""
+    elements of one CTA of 304 or more, whole slices of 128, and one sum per k-group.  That bound
+    allows for a slice left out, so whole numbers are compared exactly as well."""
     rf = cuda_lib
     P = torch.randn(F, E, generator=torch.Generator(device=DEV).manual_seed(E), device=DEV)
     G = torch.empty(F, F, dtype=torch.float64, device=DEV)
@@ -930,6 +948,7 @@ def test_frame_gram_long_unaligned_rows(cuda_lib, F, E):
     p = P.double()
     chain = E / 304 + 128 + 32
     assert ((G - p @ p.t()).abs() <= chain * 2.0 ** -24 * (p.abs() @ p.abs().t())).all()
+    _gram_of_integers(rf, F, E, 0, 0, E)
 
 
 @pytest.mark.parametrize("F,E", [(9, 300), (33, 57600), (64, 3000), (64, 60000)])
