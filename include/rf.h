@@ -319,8 +319,13 @@ rf_status rf_step_core(const uint8_t* d_mask, const uint8_t* d_cur_slot, const f
  *   d_G   fp64 [F][F] output, G[i][j] = sum_e P[i][e] * P[j][e]; the call zero-fills it on
  *         `stream` first (partial sums are added with atomics, so summation order varies
  *         between runs at the level of fp64 rounding)
- * Per-CTA partial products are fp32 (each over at most E / #SMs / 2 elements), accumulated
- * across CTAs in fp64.
+ * Products are summed in fp32 over part of a CTA's elements and in fp64 across CTAs.
+ *   - Long proxies: a CTA has its share of E among 2 or 4 CTAs per SM, at least about 384
+ *     elements, rounded up to slices of at most 128.  Each of its 4 to 32 groups of threads sums
+ *     a part of them in fp32; the groups, and pairs of CTAs, are added as unevaluated pairs of
+ *     floats (in fp64 where that leaves the range of a float).
+ *   - Short proxies, and some long ones whose rows are off the 16-byte boundaries: the fp32
+ *     sums cover all of a CTA's slices of 128 elements, at most four CTAs per SM.
  */
 rf_status rf_frame_gram(const float* d_P, int F, int64_t E, int64_t ld, double* d_G,
                         rf_stream_t stream);

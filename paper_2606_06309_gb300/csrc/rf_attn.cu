@@ -468,7 +468,7 @@ __device__ __forceinline__ void producer(const CUtensorMap* tmQ, const CUtensorM
       return true;
     };
     // the CTA's first K/V tile goes before its queries, which have to wait for the active list
-    // (4 x 64 tokens x 2 heads x 64: 8.5 -> 7.9 us per launch; block-masked launches wait for their
+    // (4 x 64 tokens x 2 heads x 64: 12.6 -> 11.2 us per launch; block-masked launches wait for their
     // tile list anyway and gained nothing)
     const int j_first = tile_first<MASKED>(u, tw, nw);
     const bool kv_first = !MASKED && k == 0;
@@ -1175,7 +1175,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 //
 // Groups of consecutive heads (item = head * pairs + pair): the queue hands out the groups one
 // after the other, so the CTAs that run together work on the heads of one group.  A group has
-// as many heads as fit their K/V in half of L2, and at least enough for six items per CTA
+// as many heads as fit their K/V in half of L2, and at least enough for four items per CTA
 // (from the active count, so on the device): one global order by cost spread the CTAs over
 // all 40 heads of a 21 x 3600-token workload (39 MB of K/V per head, 129 MB of L2) and was 5%
 // slower than no order at all, while one head per group left 13 x 1560 tokens (80 items per

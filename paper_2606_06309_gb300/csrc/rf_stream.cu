@@ -336,8 +336,8 @@ __global__ void __launch_bounds__(kKvThreads)
 // launches of their own (compaction, latents, keys and values before the attention, the Euler
 // update after it) they cost the launch, ramp and drain of each: keyframe-only step of
 // 13 x 1560 x 1536, 2.9 + 5.4 + 47 + 4.5 us in kernels, 44 us as one; four steps of 4 x 64 tokens
-// replayed as a graph, 90.2 -> 71.7 us with the copies around it; a step of them from the host
-// 33.4 -> 23.4 us (21.6 us on another box).
+// replayed as a graph, 106.9 -> 86.4 us with the copies around it; a step of them from the host
+// 57.4 -> 23.8 us.
 // ---------------------------------------------------------------------------------------
 constexpr int kTokChunk = 16 * kKvThreads;
 constexpr int kFrontTiles = kMaxFrames / kKvThreads;  // mask tiles of one thread's register

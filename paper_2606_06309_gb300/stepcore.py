@@ -136,7 +136,7 @@ class StepCore:
         frames' rows of K and V are overwritten with their projection before the attention.
 
         One call and two launches: all but the attention in the first.  4 x 64 tokens, 2 heads:
-        23.4 us per step (host and launches) against 33.4 as five calls.  Where compact, project,
+        23.8 us per step (host and launches) against 57.4 as five calls.  Where compact, project,
         project_kv, attn or step has been replaced, in a subclass or on the object, the five are
         called instead."""
         if self._own_parts():
