@@ -335,7 +335,10 @@ __global__ void __launch_bounds__(kGramThreads)
 }
 
 // Whether gram_short_kernel is the faster of the two.  On short proxies gram_kernel's clusters, its
-// wider tiles' fewer threads and its sums cost more than one atomic per entry and CTA.  Short / long,
+// wider tiles' fewer threads and its sums cost more than one atomic per entry and CTA.
+// gram_short_kernel's time grows with its CTAs, one per 128 elements (33 frames: about 5.6 us and
+// 0.36 us per 1000 elements); gram_kernel's hardly does until its CTAs have more than their 384
+// elements, and its level rises with the frames.  The lines lie where the two meet.  Short / long,
 // in us: 1 x 24000 7.3 / 8.4, 46000 8.4 / 8.3; 13 x 10001 8.4 / 10.4, 24960 14.4 / 10.4; 33 x 12000
 // 9.9 / 12.5, 24000 14.2 / 13.0, 27001 14.7 / 14.4, 57600 26.0 / 15.2; 56 x 20000 16.3 / 16.7, 30000
 // 18.2 / 17.1; 64 x 2475 10.0 / 27.5, 30000 18.9 / 23.5, 42000 28.4 / 24.3.
